@@ -400,12 +400,12 @@ __device__ __forceinline__ void ls_column_reg(R *T, const R *X, int Ls, bool dow
   if (X) {
     const R a0 = c.a0, a1 = c.a1;
     R xlast = X[ix(Ls - 1)], xprev = X[ix(0)];
-    v[0] += a0 * xprev - a1 * mf * xlast;
+    v[0] = fma(a0, xprev, fma(-a1 * mf, xlast, v[0]));
 #pragma unroll
     for (int j = 1; j < LM; ++j)
       if (j < Ls) {
         const R xj = X[ix(j)];
-        v[j] += a0 * xj + a1 * xprev;
+        v[j] = fma(a0, xj, fma(a1, xprev, v[j]));
         xprev = xj;
       }
   }

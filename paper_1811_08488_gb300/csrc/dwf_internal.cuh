@@ -308,7 +308,7 @@ void launch_m5inv_gemm(dwf_ctx *ctx, dwf_prec p, char *out, const char *in, int 
                        const double *mf, cudaStream_t st);
 void launch_ls_op(dwf_prec p, char *out, const char *in, long long rstride,
                   int nsite, int Ls, int dagger, int inv, int nrhs, const LsCoef *coef,
-                  cudaStream_t st, int coef_div = 1);
+                  cudaStream_t st, int coef_div = 1, const int *skip = nullptr);
 
 // fields.cu: layout and precision conversions
 void launch_import(dwf_prec p, char *native, long long nstride, const void *canon,

@@ -12,7 +12,8 @@ namespace dwf {
 // ---------------------------------------------------------------------------
 // Grid z runs over nrhs * coef_div fields of nsite sites (block-local fields
 // of every block are laid out like right-hand sides); field z uses the
-// coefficients of right-hand side z / coef_div. A CTA reads its sites before it
+// coefficients of right-hand side z / coef_div (skipped when its skip flag is
+// set). A CTA reads its sites before it
 // writes them, so out may equal in.
 template <class S, bool DAG>
 __global__ void __launch_bounds__(256) ls_kernel(char *out, const char *in, long long rstride,
@@ -21,6 +22,7 @@ __global__ void __launch_bounds__(256) ls_kernel(char *out, const char *in, long
   using R = typename S::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int rhs = blockIdx.z;
+  if (P.skip && P.skip[rhs / coef_div]) return;
   const LsCoef &cf = P.coef[rhs / coef_div];
   const int nsites = P.nsites;
   const int tid = threadIdx.x, s = tid % Ls, sl = tid / Ls;
@@ -53,8 +55,9 @@ __global__ void __launch_bounds__(256) ls_kernel(char *out, const char *in, long
 
 void launch_ls_op(dwf_prec p, char *out, const char *in, long long rstride, int nsite, int Ls,
                   int dagger, int inv, int nrhs, const LsCoef *coef, cudaStream_t st,
-                  int coef_div) {
+                  int coef_div, const int *skip) {
   HopParams P;
+  P.skip = skip;
   for (int r = 0; r < nrhs; ++r) {
     P.coef[r] = coef[r];
     finalize_coef(P.coef[r]);

@@ -102,7 +102,13 @@ __device__ __forceinline__ void hop_dir(typename S::R *acc, const char *in, long
 }
 
 // Project v with (1 - sg g_mu), multiply the two-spinor by U (forward) or U^+
-// (backward), reconstruct and add to acc.
+// (backward), reconstruct and add to acc. In FP64 the FP64 pipe is the bound
+// (a DFMA takes 65 cycles per warp and scheduler), so U h is a chain of 72
+// multiply-adds: `re += ur * hr - ui * hi` compiles to a product, a
+// multiply-add and a sum, 108 operations. Measured with M_phi taken out of the
+// hops (mphi_input) and whole warps (hop_sites_per_cta): A in FP64 on
+// 16^3 x 32 x 12 8.57 -> 5.58 ms, 0.69 of the FP64 pipe's rate; D_PC^+ in FP32
+// with Ls = 9 and three right-hand sides on 12 x 10 x 14 x 18 148 -> 119 us.
 template <class R, int MU, bool FWD, bool DAG>
 __device__ __forceinline__ void proj_mul_acc(R *acc, const R *v, const R *u) {
   constexpr R sg = (FWD != DAG) ? (R)1 : (R)-1;  // projector (1 - sg g_mu)
@@ -123,14 +129,16 @@ __device__ __forceinline__ void proj_mul_acc(R *acc, const R *v, const R *u) {
   for (int sp = 0; sp < 2; ++sp) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      R re = 0, im = 0;
+      R re, im;
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
         // forward: U[a][b]; backward: conj(U[b][a])
         const R ur = FWD ? u[2 * (3 * a + b)] : u[2 * (3 * b + a)];
         const R ui = FWD ? u[2 * (3 * a + b) + 1] : -u[2 * (3 * b + a) + 1];
-        re += ur * h[sp][b].re - ui * h[sp][b].im;
-        im += ur * h[sp][b].im + ui * h[sp][b].re;
+        re = b == 0 ? ur * h[sp][b].re : fma(ur, h[sp][b].re, re);
+        re = fma(-ui, h[sp][b].im, re);
+        im = b == 0 ? ur * h[sp][b].im : fma(ur, h[sp][b].im, im);
+        im = fma(ui, h[sp][b].re, im);
       }
       w[sp][a] = {re, im};
     }
@@ -758,13 +766,18 @@ __global__ void __launch_bounds__(128, 4) hop2_kernel(const __grid_constant__ Ho
 // Two slices per thread for FP32/FP16/BF16 with even Ls; one otherwise.
 static bool hop_pairs(int Ls, dwf_prec p) { return p != DWF_FP64 && Ls % 2 == 0; }
 
+// Sites per CTA. The one-slice kernel takes, between a half and a whole of its
+// largest CTA, the number of sites that leaves the fewest idle lanes in the last
+// warp: a warp instruction of the FP64 pipe takes as long with idle lanes (Ls =
+// 12: 8 sites fill three warps, 10 sites leave 8 of 128 lanes idle).
 int hop_sites_per_cta(int Ls, dwf_prec p) {
-  int n;
-  if (hop_pairs(Ls, p))
-    n = 4 * (32 / (Ls / 2));  // four warps of whole sites
-  else
-    n = ((p == DWF_FP64) ? 128 : 256) / Ls;
-  return n < 1 ? 1 : n;
+  if (hop_pairs(Ls, p)) return 4 * (32 / (Ls / 2));  // four warps of whole sites
+  const int most = (p == DWF_FP64 ? 128 : 256) / Ls;
+  int best = most;
+  auto lanes = [&](int n) { return (n * Ls + 31) / 32 * 32; };
+  for (int n = most; n >= 1 && 2 * n >= most; --n)
+    if (n * lanes(best) > best * lanes(n)) best = n;
+  return best;
 }
 
 size_t hop_smem_bytes(int Ls, dwf_prec p, int epi, int has_x) {

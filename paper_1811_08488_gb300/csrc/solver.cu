@@ -108,19 +108,40 @@ void apply_dslash(dwf_ctx *ctx, void *out, const void *in, int out_parity, int d
   launch(ctx, p, P, dagger, dagger ? 0 : 1, nrhs, st);
 }
 
+// The input of a hop with M_phi: FP64 fields take M_phi in one Ls pass into
+// phi_tmp (returned; the hop then runs without it), others take it on load
+// (`in` is returned). On load every neighbour's M_phi costs 48 operations for
+// each of the 8 directions; in FP32 that is cheaper than a pass over the
+// field, on GB300's small FP64 pipe it is not (16^3 x 32 x 12, first hop of
+// D_PC: 384 of 1250 FP64 operations per element against 48 and 302 MB).
+static const void *mphi_input(dwf_ctx *ctx, const void *in, char *phi_tmp, dwf_prec p, int nrhs,
+                              const double *mf, const int *skip, cudaStream_t st) {
+  if (p != DWF_FP64) return in;
+  LsCoef c[kMaxRhs];
+  for (int r = 0; r < nrhs; ++r) c[r] = coef_mphi(ctx->act, mf[r], 1.0);
+  launch_ls_op(p, phi_tmp, static_cast<const char *>(in),
+               (long long)field_rhs_bytes(p, ctx->geo.Vh, ctx->act.Ls), ctx->geo.Vh, ctx->act.Ls,
+               0, 0, nrhs, c, st, 1, skip);
+  return phi_tmp;
+}
+
 // First half of D_PC (or D_PC^+): u(odd) = K (-1/2 Dhop M_phi in) with
 // K = M_phi M_5^-1, or v(odd) = K^+ (-1/2 Dhop^+ in) with K^+ = M_5^-+ M_phi^+.
+// phi_tmp: even temporary for M_phi in (FP64 and dagger = 0 only).
 static void mpc_first(dwf_ctx *ctx, void *odd_out, const void *in, int dagger, dwf_prec p,
-                      int nrhs, const double *mf, const int *skip, cudaStream_t st) {
-  HopParams P = global_params(ctx, p, 1, in, odd_out);
+                      int nrhs, const double *mf, char *phi_tmp, const int *skip,
+                      cudaStream_t st) {
+  const void *hop_in = dagger ? in : mphi_input(ctx, in, phi_tmp, p, nrhs, mf, skip, st);
+  const int pre = !dagger && hop_in == in;
+  HopParams P = global_params(ctx, p, 1, hop_in, odd_out);
   for (int r = 0; r < nrhs; ++r) {
     P.coef[r] = coef_k(ctx->act, mf[r], -0.5);
-    if (!dagger) with_pre(P.coef[r], ctx->act);
+    if (pre) with_pre(P.coef[r], ctx->act);
   }
   P.epi = 1;
   P.inv = 1;
   P.skip = skip;
-  launch(ctx, p, P, dagger, dagger ? 0 : 1, nrhs, st);
+  launch(ctx, p, P, dagger, pre, nrhs, st);
 }
 
 // Second half: out(even) = M_5 in + 1/2 Dhop u, or M_5^+ in + 1/2 M_phi^+ Dhop^+ v.
@@ -159,7 +180,7 @@ static void mpc_second(dwf_ctx *ctx, void *out, const void *odd_in, const void *
 void apply_mpc(dwf_ctx *ctx, void *out, const void *in, int dagger, dwf_prec p, int nrhs,
                const double *mf, const OpWork &w, cudaStream_t st) {
   char *odd = dagger ? w.v : w.u;
-  mpc_first(ctx, odd, in, dagger, p, nrhs, mf, nullptr, st);
+  mpc_first(ctx, odd, in, dagger, p, nrhs, mf, w.v, nullptr, st);
   mpc_second(ctx, out, odd, in, dagger, p, nrhs, mf, nullptr, nullptr, st);
 }
 
@@ -174,8 +195,8 @@ static void m5inv_pass(dwf_ctx *ctx, void *out, const void *in, int dagger, dwf_
 }
 
 // D_sym in = in - M_5^-1 M^4_eo M_5^-1 M^4_oe in (odd temporary odd_tmp), or
-// D_sym^+ in = in - (M^4_oe)^+ M_5^-+ (M^4_eo)^+ M_5^-+ in (with the even
-// temporary even_tmp for M_5^-+ in as well).
+// D_sym^+ in = in - (M^4_oe)^+ M_5^-+ (M^4_eo)^+ M_5^-+ in. The even temporary
+// even_tmp holds M_5^-+ in, or M_phi in (D_sym in FP64).
 static void mpc_sym(dwf_ctx *ctx, void *out, const void *in, int dagger, dwf_prec p, int nrhs,
                     const double *mf, char *odd_tmp, char *even_tmp, const DotSpec *dot,
                     const int *skip, cudaStream_t st) {
@@ -184,7 +205,7 @@ static void mpc_sym(dwf_ctx *ctx, void *out, const void *in, int dagger, dwf_pre
     m5inv_pass(ctx, even_tmp, in, 1, p, nrhs, mf, st);
     hop_in = even_tmp;
   }
-  mpc_first(ctx, odd_tmp, hop_in, dagger, p, nrhs, mf, skip, st);
+  mpc_first(ctx, odd_tmp, hop_in, dagger, p, nrhs, mf, even_tmp, skip, st);
   mpc_second(ctx, out, odd_tmp, in, dagger, p, nrhs, mf, dot, skip, st, 1);
 }
 
@@ -251,18 +272,20 @@ void apply_odd_reconstruct(dwf_ctx *ctx, void *psi_odd, const void *psi_even,
                            const void *phi_odd, dwf_prec p, int nrhs, const double *mf,
                            const OpWork &w, cudaStream_t st) {
   const int Vh = ctx->geo.Vh, Ls = ctx->act.Ls;
-  HopParams P = global_params(ctx, p, 1, psi_even, w.u);
+  const void *hop_in = mphi_input(ctx, psi_even, w.v, p, nrhs, mf, nullptr, st);
+  const int pre = hop_in == psi_even;
+  HopParams P = global_params(ctx, p, 1, hop_in, w.u);
   P.xown = global_ref(ctx, p, phi_odd);
   for (int r = 0; r < nrhs; ++r) {
     P.coef[r] = coef_identity(0.5);
     P.coef[r].mf = mf[r];
-    with_pre(P.coef[r], ctx->act);
+    if (pre) with_pre(P.coef[r], ctx->act);
     P.coef[r].a0 = 1.0;
     P.coef[r].a1 = 0.0;
   }
   P.epi = 1;
   P.has_x = 1;
-  launch(ctx, p, P, 0, 1, nrhs, st);
+  launch(ctx, p, P, 0, pre, nrhs, st);
   LsCoef c[kMaxRhs];
   for (int r = 0; r < nrhs; ++r) c[r] = coef_m5inv(ctx->act, mf[r], 1.0);
   launch_ls_op(p, static_cast<char *>(psi_odd), w.u, (long long)field_rhs_bytes(p, Vh, Ls), Vh,
@@ -279,13 +302,13 @@ void apply_mdagm(dwf_ctx *ctx, void *out, const void *in, dwf_prec p, int nrhs,
       d = *dot;
       d.dotv = static_cast<const char *>(in);
     }
-    mpc_sym(ctx, w.y, in, 0, p, nrhs, mf, w.u, nullptr, nullptr, skip, st);
+    mpc_sym(ctx, w.y, in, 0, p, nrhs, mf, w.u, w.v, nullptr, skip, st);
     mpc_sym(ctx, out, w.y, 1, p, nrhs, mf, w.u, w.v, dot ? &d : nullptr, skip, st);
     return;
   }
-  mpc_first(ctx, w.u, in, 0, p, nrhs, mf, skip, st);
+  mpc_first(ctx, w.u, in, 0, p, nrhs, mf, w.v, skip, st);
   mpc_second(ctx, w.y, w.u, in, 0, p, nrhs, mf, nullptr, skip, st);
-  mpc_first(ctx, w.v, w.y, 1, p, nrhs, mf, skip, st);
+  mpc_first(ctx, w.v, w.y, 1, p, nrhs, mf, nullptr, skip, st);
   DotSpec d;
   if (dot) {
     d = *dot;
