@@ -295,47 +295,55 @@ __device__ __forceinline__ void reconstruct_row2(R *u, R sg) {
   }
 }
 
+// One word (or its start) of a link record in global or shared memory.
+template <bool SMEM, class T>
+__device__ __forceinline__ T ldl(const T *p) {
+  if constexpr (SMEM) return *p;
+  else return __ldg(p);
+}
+
 // Load the link record whose word 0 is at w; word k is at w[k * ws] (the
 // chunk-major link layout: ws = number of link owners). recon: the record
-// holds two rows and a sign (reconstruct-12, FP32/FP16/BF16 only).
-template <class S>
+// holds two rows and a sign (reconstruct-12, FP32/FP16/BF16 only). SMEM: the
+// record is in shared memory.
+template <class S, bool SMEM = false>
 __device__ __forceinline__ void load_link(const uint4 *w, size_t ws, typename S::R *u,
                                           int recon = 0) {
   if constexpr (std::is_same<S, F64>::value) {
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-      const double2 q = __ldg(reinterpret_cast<const double2 *>(w + k * ws));
+      const double2 q = ldl<SMEM>(reinterpret_cast<const double2 *>(w + k * ws));
       u[2 * k] = q.x; u[2 * k + 1] = q.y;
     }
   } else if constexpr (std::is_same<S, F32>::value) {
     if (recon) {
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        const float4 q = __ldg(reinterpret_cast<const float4 *>(w + k * ws));
+        const float4 q = ldl<SMEM>(reinterpret_cast<const float4 *>(w + k * ws));
         u[4 * k] = q.x; u[4 * k + 1] = q.y; u[4 * k + 2] = q.z; u[4 * k + 3] = q.w;
       }
-      reconstruct_row2<float>(u, __ldg(reinterpret_cast<const float *>(w + 3 * ws)));
+      reconstruct_row2<float>(u, ldl<SMEM>(reinterpret_cast<const float *>(w + 3 * ws)));
     } else {
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const float4 q = __ldg(reinterpret_cast<const float4 *>(w + k * ws));
+        const float4 q = ldl<SMEM>(reinterpret_cast<const float4 *>(w + k * ws));
         u[4 * k] = q.x; u[4 * k + 1] = q.y; u[4 * k + 2] = q.z; u[4 * k + 3] = q.w;
       }
-      const float2 q = __ldg(reinterpret_cast<const float2 *>(w + 4 * ws));
+      const float2 q = ldl<SMEM>(reinterpret_cast<const float2 *>(w + 4 * ws));
       u[16] = q.x; u[17] = q.y;
     }
   } else {
     if (recon) {
       float t[16];
-      unpack8<F16>(__ldg(w), t);
-      unpack8<F16>(__ldg(w + ws), t + 8);
+      unpack8<F16>(ldl<SMEM>(w), t);
+      unpack8<F16>(ldl<SMEM>(w + ws), t + 8);
 #pragma unroll
       for (int k = 0; k < 12; ++k) u[k] = t[k];
       reconstruct_row2<float>(u, t[12]);
     } else {
       float t[24];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) unpack8<F16>(__ldg(w + k * ws), t + 8 * k);
+      for (int k = 0; k < 3; ++k) unpack8<F16>(ldl<SMEM>(w + k * ws), t + 8 * k);
 #pragma unroll
       for (int k = 0; k < 18; ++k) u[k] = t[k];
     }

@@ -155,6 +155,10 @@ struct HopParams {
   const int *nbr = nullptr;  // [n_out][8], direction 2*mu + (0 fwd, 1 bwd)
   int n_out = 0;             // output sites per block
   int in_limit = 0;          // inputs with index >= in_limit are zero
+  int n_dense = 0;           // sites below it run all eight directions (see dense_sites),
+  const int *nbr_read = nullptr;  // reading these neighbours (nbr with the absent ones replaced)
+  int site_off = 0;          // first output site of the launch (set by the launcher)
+  int dirs = 0xff;           // all eight directions (the dense FP32 hop branches on it)
   int xown_limit = 0;        // xown is zero for sites >= xown_limit
   int out_link_off = 0;      // combined link id of output site i: off + i
   int in_link_off = 0;
@@ -172,6 +176,7 @@ struct HopParams {
   unsigned int *counters = nullptr;  // [rhs][block]
   const int *skip = nullptr;    // per rhs: nonzero = skip (converged)
   const int *bskip = nullptr;   // per (rhs, block): nonzero = skip (inner stop met)
+  int prof_again = 0;           // 1: a further launch of the same hop (set by the launcher)
   KernProf *prof = nullptr;     // timer slot of this launch (null: profiling off)
   unsigned long long alg_bytes = 0;  // compulsory bytes of this launch
   LsCoef coef[kMaxRhs];
@@ -199,6 +204,10 @@ struct BlockGeometry {
   std::vector<int> nbr_oe;  // [n_o1][8]: odd out <- even in (local even index or -1)
   std::vector<int> nbr_eo;  // [n_e2][8]: even out <- odd in (local odd index or -1)
   std::vector<int> gsite;   // [nblocks][n_comb] global lexicographic site of each owner
+  // leading sites of each block hop with all or most neighbours [snake][hop 1..4], and
+  // their neighbours with the absent ones replaced (empty where none is absent)
+  int dense[2][4];
+  std::vector<int> nbr_read[2][4];
   std::vector<int> gmap_b;  // [nblocks][n_b] global even half index of block sites
 };
 
@@ -300,7 +309,7 @@ namespace dwf {
 template <class S>
 void launch_hop(const HopParams &P, int dagger, int pre_mphi, int nrhs, cudaStream_t st);
 int hop_sites_per_cta(int Ls, dwf_prec p);
-size_t hop_smem_bytes(int Ls, dwf_prec p, int epi, int has_x);
+size_t hop_smem_bytes(int Ls, dwf_prec p, int epi, int has_x, int recon);
 
 // ls.cu: Ls-local operators (M_5, M_5^-1) on native fields
 // Tensor-core M_5^-1 (csrc/m5tc.cu); synchronises `st` and checks the status word.

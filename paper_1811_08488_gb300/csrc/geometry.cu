@@ -59,6 +59,43 @@ static inline int side1(int u, int bl, int L) {
   return (u - bl + 1 <= L - u) ? 1 : 2;
 }
 
+// How many of the leading n_out sites run all eight directions of a block hop: ring
+// after ring (the sites at distance 0, 1, 2 end at `ends`) as long as a ring's sites
+// have 5 of 8 neighbours or more on average. A direction that is left out saves its
+// arithmetic, one that always runs is loaded ahead of it. In 12^3 x 16 blocks the
+// even sites at distance 0, 1 and 2 have 8, 7 and 1 to 2 odd neighbours in the
+// region (FP16 hop 2: 427 us with all sites run by tests, 418 with distance 0 run
+// densely). In 2^4 blocks every site has 4 of its own block.
+// read: the neighbours with the absent ones replaced by another of the site's
+// (left empty when none is absent).
+static int dense_sites(const std::vector<int> &nbr, int n_out, std::array<int, 3> ends,
+                       int in_limit, std::vector<int> &read) {
+  auto has = [&](size_t i) { return nbr[i] >= 0 && nbr[i] < in_limit; };
+  auto count = [&](int from, int to) {
+    long long have = 0;
+    for (size_t i = (size_t)from * 8; i < (size_t)to * 8; ++i) have += has(i);
+    return have;
+  };
+  int n = 0;
+  for (int e : ends) {
+    e = std::min(e, n_out);
+    if (e <= n) continue;
+    if (count(n, e) < 5LL * (e - n)) break;
+    n = e;
+  }
+  // whole CTAs of sites are run, so the table covers all
+  if (n == 0 || count(0, n_out) == 8LL * n_out) return n;
+  read.assign(nbr.begin(), nbr.begin() + (size_t)n_out * 8);
+  for (size_t s = 0; s < (size_t)n_out; ++s) {
+    int some = 0;
+    for (int k = 0; k < 8; ++k)
+      if (has(8 * s + k)) some = nbr[8 * s + k];
+    for (int k = 0; k < 8; ++k)
+      if (!has(8 * s + k)) read[8 * s + k] = some;
+  }
+  return n;
+}
+
 void build_block_geometry(BlockGeometry &bg, const int dims[4], const int block[4]) {
   int nb[4];
   for (int m = 0; m < 4; ++m) {
@@ -145,6 +182,15 @@ void build_block_geometry(BlockGeometry &bg, const int dims[4], const int block[
         auto it = od_idx.find(nb_lex(ev[i], mu, dir));
         if (it != od_idx.end()) bg.nbr_eo[(size_t)i * 8 + 2 * mu + dir] = it->second;
       }
+
+  for (int snake = 0; snake < 2; ++snake) {
+    const int no = snake ? bg.n_o1 : bg.n_ob, ne = snake ? bg.n_e2 : bg.n_b;
+    const std::array<int, 3> odd = {bg.n_ob, bg.n_o1, bg.n_o1}, even = {bg.n_b, bg.n_e1, bg.n_e2};
+    bg.dense[snake][0] = dense_sites(bg.nbr_oe, no, odd, bg.n_b, bg.nbr_read[snake][0]);
+    bg.dense[snake][1] = dense_sites(bg.nbr_eo, ne, even, no, bg.nbr_read[snake][1]);
+    bg.dense[snake][2] = dense_sites(bg.nbr_oe, no, odd, ne, bg.nbr_read[snake][2]);
+    bg.dense[snake][3] = dense_sites(bg.nbr_eo, bg.n_b, even, no, bg.nbr_read[snake][3]);
+  }
 
   bg.gsite.assign((size_t)bg.nblocks * bg.n_comb, 0);
   bg.gmap_b.assign((size_t)bg.nblocks * bg.n_b, 0);

@@ -4,15 +4,37 @@
 //
 // Two kernels. hop2_kernel (FP32/FP16/BF16 fields, even Ls): one thread per
 // pair of slices (s0, s0 + 1) of one output site; the Ls/2 threads of a site
-// are consecutive lanes of one warp (a warp holds whole sites), so the links
-// of a site are loaded once per warp line, and everything that couples
-// neighbouring slices -- M_phi on load (s0 - 1, s0 + 2), the Ls epilogue
-// (M_phi^+, M_5^-1, K = M_phi M_5^-1 and their adjoints) and the x-term of the
-// epilogue -- is exchanged between those lanes with warp shuffles; the
-// epilogue's (1 - r S)^-1 is a scan over the site's lanes. It uses no shared
-// memory outside its reductions, so the unified L1 serves the neighbour
-// gather. hop_kernel (FP64 fields, odd Ls): one thread per output (site, s),
-// the Ls epilogue walks columns in shared memory.
+// are consecutive lanes of one warp (a warp holds whole sites), and everything
+// that couples neighbouring slices -- M_phi on load (s0 - 1, s0 + 2), the Ls
+// epilogue (M_phi^+, M_5^-1, K = M_phi M_5^-1 and their adjoints) and the x-term
+// of the epilogue -- is exchanged between those lanes with warp shuffles; the
+// epilogue's (1 - r S)^-1 is a scan over the site's lanes.
+//
+// What bounds hop2_kernel: 16 warps per SM (48 accumulators a thread) waiting for
+// the gather, 8 x 96 bytes per element in FP32 through L2 (gather and stores alone:
+// 318 us on 24^3 x 64 x 16, FP32 adjoint). Two things shorten the wait:
+// - The links are staged in shared memory once per CTA. Read by every lane of a
+//   site they were 5 of the 11 loads of a direction for 1/20 of its bytes, and
+//   without them the adjoint hop took 353 us instead of 513.
+// - The next direction's spinors are loaded into the registers that the projection
+//   has just freed, while the projected spins are multiplied by the link.
+// And the Ls epilogue's scan runs one step over all 24 components at a time, with
+// shared factors, 480 instead of about 1100 instructions per thread.
+// Measured on 24^3 x 64 x 16, before -> after: FP32 M^4 613 -> 533 us, adjoint
+// 513 -> 410, FP16 642 -> 486 and 433 -> 384, A in FP32 2547 -> 2072. Not kept:
+// rings of stages in shared memory filled by cp.async or by TMA boxes, all
+// bit-identical: the work to issue them (150 instructions a direction beside 230 of
+// arithmetic) and the larger code cost more than the waiting they save (853 and
+// 883 us for FP32 M^4); mma.m16n8k16 for FP16 fields (one site per warp: 968
+// instructions per site instead of 553, 660 us for the adjoint); an L2 prefetch
+// of the rows that come next (535 us).
+//
+// A launch runs `dense` sites, which have all or most neighbours, in this form.
+// A block's outer ring, with one or two neighbours each, runs direction by
+// direction with the links read where they are (DENSE = false).
+//
+// hop_kernel (FP64 fields, odd Ls): one thread per output (site, s), the Ls
+// epilogue walks columns in shared memory.
 //
 // For output site x and direction mu (chiral basis, g_mu = [[0, A],[A^+, 0]]):
 //   forward : (1 - sg g_mu) U_mu(x)      chi(x+mu)
@@ -22,6 +44,7 @@
 // With PRE, the input is chi = M_phi psi = b psi + c C psi, formed on load:
 // chi_u(s) = b psi_u(s) + c psi_u(s-1), chi_l(s) = b psi_l(s) + c psi_l(s+1),
 // with the wrap factor -m_f.
+#include <algorithm>
 #include <type_traits>
 
 #include "device_common.cuh"
@@ -258,7 +281,7 @@ __device__ __noinline__ void prof_exit(const HopParams &P) {
   const unsigned long long t1 = gtimer_ns();
   const unsigned long long t0 = *reinterpret_cast<volatile unsigned long long *>(&k->start);
   k->total_ns += t1 - t0;
-  k->launches += 1;
+  if (!P.prof_again) k->launches += 1;
   k->bytes += P.alg_bytes;
   k->done = 0;
   __threadfence();
@@ -355,7 +378,7 @@ __global__ void __launch_bounds__(256) hop_kernel(const __grid_constant__ HopPar
 // Two slices per thread: thread (site, s0 = 2j) computes s0 and s0 + 1. Chunk c
 // of both slices is one 32-byte word, so every spinor load and store is a
 // 256-bit access and a warp moves one contiguous kilobyte per instruction; the
-// link is loaded once for both slices; with M_phi on load, the two slices
+// link serves both slices; with M_phi on load, the two slices
 // supply each other's s -> s +- 1 neighbours and only the outer two halves
 // (s0 - 1 upper, s0 + 2 lower) are loaded in addition. Arithmetic runs on
 // float2 pairs (slice s0, slice s0 + 1) with Blackwell's packed FP32
@@ -403,25 +426,34 @@ __device__ __forceinline__ C2 add_phase_s(C2 x, C2 z, float2 sp, float2 sn) {
   else return {fma_s(x.re, z.im, a), fma_s(x.im, z.re, b)};
 }
 
-// Packed counterpart of proj_mul_acc: v, acc hold 24 reals of both slices.
-// SCALED: v holds stored FP16/BF16 values whose per-slice scales sc are
-// applied in the accumulation (the projector and U are linear).
-template <int MU, bool FWD, bool DAG, bool SCALED = false>
-__device__ __forceinline__ void proj_mul_acc2(float2 *acc, const float2 *v, const float *u,
-                                              float2 sc = make_float2(1.f, 1.f)) {
+// Packed counterpart of proj_mul_acc in two parts; v, h and acc hold both slices.
+// h = (1 - SG g_mu) v, the two projected spins.
+struct HalfSpinor {
+  C2 h[2][3];
+};
+template <int MU, bool FWD, bool DAG>
+__device__ __forceinline__ void project2(HalfSpinor &p, const float2 *v) {
   constexpr int SG = (FWD != DAG) ? 1 : -1;  // projector (1 - SG g_mu)
   using A = ProjA<MU>;
-  using Ad = ProjAd<MU>;
-  C2 h[2][3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const C2 vu0{v[0 * 6 + 2 * c], v[0 * 6 + 2 * c + 1]};
     const C2 vu1{v[1 * 6 + 2 * c], v[1 * 6 + 2 * c + 1]};
     const C2 vl[2] = {{v[2 * 6 + 2 * c], v[2 * 6 + 2 * c + 1]},
                       {v[3 * 6 + 2 * c], v[3 * 6 + 2 * c + 1]}};
-    h[0][c] = add_phase<A::p0, -SG>(vu0, vl[A::s0]);
-    h[1][c] = add_phase<A::p1, -SG>(vu1, vl[A::s1]);
+    p.h[0][c] = add_phase<A::p0, -SG>(vu0, vl[A::s0]);
+    p.h[1][c] = add_phase<A::p1, -SG>(vu1, vl[A::s1]);
   }
+}
+// acc += the spinor reconstructed from U h (U^+ h backward). SCALED: h came from
+// stored FP16/BF16 values whose per-slice scales sc are applied in the
+// accumulation (the projector and U are linear).
+template <int MU, bool FWD, bool DAG, bool SCALED = false>
+__device__ __forceinline__ void mul_acc2(float2 *acc, const HalfSpinor &p, const float *u,
+                                         float2 sc = make_float2(1.f, 1.f)) {
+  constexpr int SG = (FWD != DAG) ? 1 : -1;
+  using Ad = ProjAd<MU>;
+  const float2 scn = make_float2(-sc.x, -sc.y);
   C2 w[2][3];
 #pragma unroll
   for (int sp = 0; sp < 2; ++sp) {
@@ -433,15 +465,14 @@ __device__ __forceinline__ void proj_mul_acc2(float2 *acc, const float2 *v, cons
         // forward: U[a][b]; backward: conj(U[b][a])
         const float ur = FWD ? u[2 * (3 * a + b)] : u[2 * (3 * b + a)];
         const float ui = FWD ? u[2 * (3 * a + b) + 1] : -u[2 * (3 * b + a) + 1];
-        re = __ffma2_rn(bc(ur), h[sp][b].re, re);
-        re = __ffma2_rn(bc(-ui), h[sp][b].im, re);
-        im = __ffma2_rn(bc(ur), h[sp][b].im, im);
-        im = __ffma2_rn(bc(ui), h[sp][b].re, im);
+        re = __ffma2_rn(bc(ur), p.h[sp][b].re, re);
+        re = __ffma2_rn(bc(-ui), p.h[sp][b].im, re);
+        im = __ffma2_rn(bc(ur), p.h[sp][b].im, im);
+        im = __ffma2_rn(bc(ui), p.h[sp][b].re, im);
       }
       w[sp][a] = {re, im};
     }
   }
-  const float2 scn = make_float2(-sc.x, -sc.y);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     if constexpr (SCALED) {
@@ -481,80 +512,122 @@ struct PairLanes {
   float fm, fp;     // their wrap factors (-m_f across the Ls boundary, else 1)
 };
 
-template <class S, int MU, bool FWD, bool DAG, bool PRE, bool RC>
-__device__ __forceinline__ void hop_dir2(float2 *acc, const char *in, long long soff, int cs,
-                                         int j, bool valid, int s0, int Ls, const uint4 *lk,
-                                         size_t ls, const LsCoef &cf, const PairLanes &pl) {
-  float2 v[24];
-  constexpr bool kFold = !PRE && !std::is_same<S, F32>::value;  // scales folded into the FMAs
-  float2 sc = make_float2(1.f, 1.f);
-  {
-    float v0[24], v1[24];
-    if (valid) {
-      if constexpr (kFold)
-        load24x2_unscaled<S>(in, soff, cs, j * Ls + s0, v0, v1, sc);
-      else
-        load24x2<S>(in, soff, cs, j * Ls + s0, v0, v1);
+// ---------------------------------------------------------------------------
+// Links in shared memory. The Ls/2 lanes of a site all need its 8 links; read from
+// global memory by each lane they cost as many L1 requests as the spinors for a
+// twentieth of the bytes. The CTA copies the links of its sites once, 16
+// bytes per lane, to [direction][word][site] and every lane reads them from there.
+// ---------------------------------------------------------------------------
+template <class S, bool RC> __host__ __device__ constexpr int link_words() {
+  return RC ? S::kLinkChunksRecon : S::kLinkChunks;
+}
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src)
+               : "memory");
+}
+// Start the copy (128 threads). An absent neighbour's link is zero. FP16 records are widened to the FP32 record on the way, once per link instead of by
+// each of the site's lanes (conversions run on the FMA pipe, 8 x 18 of them per
+// lane otherwise).
+template <class S, bool RC>
+__device__ __forceinline__ void stage_links(uint4 *sl, const HopParams &P, const uint4 *links,
+                                            int site0) {
+  constexpr int LC = link_words<S, RC>(), LS = link_words<F32, RC>();
+  const size_t ls = (size_t)P.link_cs;
+  for (int e = threadIdx.x; e < 8 * P.nsites; e += 128) {
+    const int d = e / P.nsites, i = e - d * P.nsites, site = site0 + i;
+    if (site >= P.n_out) continue;
+    const uint4 *lmu = links + (size_t)(d >> 1) * LC * ls;
+    uint4 *dst = sl + d * LS * P.nsites;
+    const int j = __ldg(P.nbr + (size_t)site * 8 + d);
+    if ((unsigned)j >= (unsigned)P.in_limit) {
+#pragma unroll
+      for (int w = 0; w < LS; ++w) dst[w * P.nsites + i] = make_uint4(0u, 0u, 0u, 0u);
+      continue;
+    }
+    const uint4 *src = lmu + ((d & 1) ? P.in_link_off + j : P.out_link_off + site);
+    if constexpr (S::kHalf) {
+      float t[8 * LC];
+#pragma unroll
+      for (int w = 0; w < LC; ++w) unpack8<F16>(__ldg(src + w * ls), t + 8 * w);
+#pragma unroll
+      for (int w = 0; w < LS; ++w)
+        dst[w * P.nsites + i] = make_uint4(__float_as_uint(t[4 * w]), __float_as_uint(t[4 * w + 1]),
+                                           __float_as_uint(t[4 * w + 2]), __float_as_uint(t[4 * w + 3]));
     } else {
 #pragma unroll
-      for (int k = 0; k < 24; ++k) v0[k] = v1[k] = 0.f;
-    }
-    if constexpr (PRE) {
-      // M_phi on both slices as packed FMAs: (chi(s0), chi(s0+1)) =
-      // b (v(s0), v(s0+1)) + c (shifted neighbours); the outer halves come
-      // from the neighbouring lanes of the same site (all lanes take part)
-      const float2 b2 = bc(cf.f.pre_b), c2 = bc(cf.f.pre_c);
-#pragma unroll
-      for (int k = 0; k < 12; ++k) {  // upper: chi(s0) <- s0-1, chi(s0+1) <- s0
-        const float w = __shfl_sync(0xffffffffu, v1[k], pl.up);
-        v[k] = __ffma2_rn(c2, make_float2(pl.fm * w, v0[k]),
-                          __fmul2_rn(b2, make_float2(v0[k], v1[k])));
-      }
-#pragma unroll
-      for (int k = 0; k < 12; ++k) {  // lower: chi(s0) <- s0+1, chi(s0+1) <- s0+2
-        const float w = __shfl_sync(0xffffffffu, v0[12 + k], pl.dn);
-        v[12 + k] = __ffma2_rn(c2, make_float2(v1[12 + k], pl.fp * w),
-                               __fmul2_rn(b2, make_float2(v0[12 + k], v1[12 + k])));
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < 24; ++k) v[k] = make_float2(v0[k], v1[k]);
+      for (int w = 0; w < LC; ++w) cp_async16(dst + w * P.nsites + i, src + w * ls);
     }
   }
-  if (valid) {
-    float u[18];
-    load_link<S>(lk, ls, u, RC ? 1 : 0);
-    proj_mul_acc2<MU, FWD, DAG, kFold>(acc, v, u, sc);
-  }
+  if constexpr (!S::kHalf) asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <class S>
+__device__ __forceinline__ void wait_links() {
+  if constexpr (!S::kHalf) asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
 }
 
-template <class S, int MU, bool DAG, bool PRE, bool RC>
-__device__ __forceinline__ void hop_mu2(float2 *acc, const HopParams &P, const char *in,
-                                        const uint4 *links, const int *nb, bool active, int site,
-                                        int s0, const LsCoef &cf, const PairLanes &pl) {
-  constexpr int LC = RC ? S::kLinkChunksRecon : S::kLinkChunks;
-  const int jf = active ? nb[2 * MU] : -1, jb = active ? nb[2 * MU + 1] : -1;
-  const size_t ls = (size_t)P.link_cs;
-  const uint4 *lmu = links + (size_t)MU * LC * ls;
-  const bool vf = jf >= 0 && jf < P.in_limit, vb = jb >= 0 && jb < P.in_limit;
+// The input of one direction as loaded (FP16/BF16 without their scales).
+struct DirIn {
+  float v0[24], v1[24];
+  float2 sc;
+};
+template <class S>
+__device__ __forceinline__ void load_dir2(DirIn &in2, const char *in, long long soff, int cs,
+                                          int e) {
+  if constexpr (S::kHalf)
+    load24x2_unscaled<S>(in, soff, cs, e, in2.v0, in2.v1, in2.sc);
+  else
+    load24x2<S>(in, soff, cs, e, in2.v0, in2.v1);
+}
+
+// The projected spins of one direction from its loaded input.
+template <class S, int MU, bool FWD, bool DAG, bool PRE>
+__device__ __forceinline__ void dir_project(HalfSpinor &h, const DirIn &d, const LsCoef &cf,
+                                            const PairLanes &pl) {
+  float2 v[24];
   if constexpr (PRE) {
-    // every lane of the warp takes part (the M_phi halves are exchanged
-    // between lanes); a direction no lane of the warp has is skipped by all
-    if (__any_sync(0xffffffffu, vf))
-      hop_dir2<S, MU, true, DAG, PRE, RC>(acc, in, P.in.scale_off, P.in.cs, jf, vf, s0, P.Ls,
-                                      lmu + P.out_link_off + site, ls, cf, pl);
-    if (__any_sync(0xffffffffu, vb))
-      hop_dir2<S, MU, false, DAG, PRE, RC>(acc, in, P.in.scale_off, P.in.cs, jb, vb, s0, P.Ls,
-                                       lmu + P.in_link_off + jb, ls, cf, pl);
+    // M_phi on both slices as packed FMAs: (chi(s0), chi(s0+1)) =
+    // b (v(s0), v(s0+1)) + c (shifted neighbours); the outer halves come
+    // from the neighbouring lanes of the same site (all lanes take part). The
+    // wrap factors and the slices' scales are folded into the coefficients.
+    const float b = cf.f.pre_b, c = cf.f.pre_c;
+    float2 bs = bc(b), cu = make_float2(c * pl.fm, c), cl = make_float2(c, c * pl.fp);
+    if constexpr (S::kHalf) {
+      const float sm = __shfl_sync(0xffffffffu, d.sc.y, pl.up);
+      const float sp = __shfl_sync(0xffffffffu, d.sc.x, pl.dn);
+      bs = make_float2(b * d.sc.x, b * d.sc.y);
+      cu = make_float2(cu.x * sm, c * d.sc.x);
+      cl = make_float2(c * d.sc.y, cl.y * sp);
+    }
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {  // upper: chi(s0) <- s0-1, chi(s0+1) <- s0
+      const float w = __shfl_sync(0xffffffffu, d.v1[k], pl.up);
+      v[k] = __ffma2_rn(cu, make_float2(w, d.v0[k]), __fmul2_rn(bs, make_float2(d.v0[k], d.v1[k])));
+    }
+#pragma unroll
+    for (int k = 12; k < 24; ++k) {  // lower: chi(s0) <- s0+1, chi(s0+1) <- s0+2
+      const float w = __shfl_sync(0xffffffffu, d.v0[k], pl.dn);
+      v[k] = __ffma2_rn(cl, make_float2(d.v1[k], w), __fmul2_rn(bs, make_float2(d.v0[k], d.v1[k])));
+    }
   } else {
-    // no exchange between lanes: each lane branches on its own neighbours
-    if (vf)
-      hop_dir2<S, MU, true, DAG, PRE, RC>(acc, in, P.in.scale_off, P.in.cs, jf, true, s0, P.Ls,
-                                      lmu + P.out_link_off + site, ls, cf, pl);
-    if (vb)
-      hop_dir2<S, MU, false, DAG, PRE, RC>(acc, in, P.in.scale_off, P.in.cs, jb, true, s0, P.Ls,
-                                       lmu + P.in_link_off + jb, ls, cf, pl);
+#pragma unroll
+    for (int k = 0; k < 24; ++k) v[k] = make_float2(d.v0[k], d.v1[k]);
   }
+  project2<MU, FWD, DAG>(h, v);
+}
+// Its contribution; lk: the site's link (STAGED: in shared memory), words ls apart.
+template <class S, int MU, bool FWD, bool DAG, bool PRE, bool RC, bool STAGED>
+__device__ __forceinline__ void dir_add(float2 *acc, const HalfSpinor &h, float2 sc, const uint4 *lk,
+                                        size_t ls) {
+  constexpr bool kFold = !PRE && S::kHalf;  // scales folded into the FMAs
+  float u[18];
+  if constexpr (STAGED)
+    load_link<F32, true>(lk, ls, u, RC ? 1 : 0);
+  else
+    load_link<S>(lk, ls, u, RC ? 1 : 0);
+  mul_acc2<MU, FWD, DAG, kFold>(acc, h, u, kFold ? sc : make_float2(1.f, 1.f));
 }
 
 // The x-term of the Ls epilogue, out += (a0 + a1 S) x, on the thread's slices
@@ -618,8 +691,9 @@ __device__ __forceinline__ void add_x_term2(float *o0, float *o1, const char *x,
 
 // EPI: the Ls epilogue is compiled in (its column registers would otherwise
 // weigh on the plain hop's register allocation).
-template <class S, bool DAG, bool PRE, bool RC, bool EPI>
+template <class S, bool DAG, bool PRE, bool RC, bool EPI, bool DENSE>
 __device__ __forceinline__ void hop2_body(const HopParams &P) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
   const int rhs = blockIdx.z, blk = blockIdx.y;
   if (P.skip && P.skip[rhs]) return;
@@ -630,7 +704,7 @@ __device__ __forceinline__ void hop2_body(const HopParams &P) {
   const int jp = lane % np, slw = lane / np;
   const int sl = (tid >> 5) * spw + slw;
   const int s0 = 2 * jp;
-  const int site0 = blockIdx.x * nsites;
+  const int site0 = P.site_off + blockIdx.x * nsites;
   const int site = site0 + sl;
   const bool active = (slw < spw) && (site < P.n_out);
   const LsCoef &cf = P.coef[rhs];
@@ -647,15 +721,91 @@ __device__ __forceinline__ void hop2_body(const HopParams &P) {
   float2 acc[24];
 #pragma unroll
   for (int k = 0; k < 24; ++k) acc[k] = make_float2(0.f, 0.f);
-  {
-    // every lane runs the direction loop (the M_phi halves are exchanged
-    // between lanes); inactive lanes load and add nothing
-    const int *nb = P.nbr + (size_t)(active ? site : 0) * 8;
-    hop_mu2<S, 0, DAG, PRE, RC>(acc, P, in, links, nb, active, site, s0, cf, pl);
-    hop_mu2<S, 1, DAG, PRE, RC>(acc, P, in, links, nb, active, site, s0, cf, pl);
-    hop_mu2<S, 2, DAG, PRE, RC>(acc, P, in, links, nb, active, site, s0, cf, pl);
-    hop_mu2<S, 3, DAG, PRE, RC>(acc, P, in, links, nb, active, site, s0, cf, pl);
+  DirIn d;
+#define HOP_LOAD(J) load_dir2<S>(d, in, P.in.scale_off, P.in.cs, (J) * Ls + s0)
+#define HOP_PROJECT(D) \
+  HalfSpinor h;        \
+  dir_project<S, (D) / 2, ((D) & 1) == 0, DAG, PRE>(h, d, cf, pl);
+  if constexpr (DENSE) {
+    // Every direction runs; where a neighbour is absent the link is zero (and
+    // nbr_read names another neighbour of the site). The next direction's spinors
+    // are loaded while this one's projected spins are multiplied (not for FP32
+    // with M_phi on load, whose registers that would spill); the links arrive while
+    // the first spinors are on their way.
+    constexpr bool kPipe = S::kHalf || !PRE;
+    constexpr int LC = link_words<F32, RC>();
+    const int *nb = P.nbr_read + (size_t)(active ? site : 0) * 8;
+    uint4 *sl_links = reinterpret_cast<uint4 *>(smem_raw);
+    stage_links<S, RC>(sl_links, P, links, site0);
+    const uint4 *lk = sl_links + min(sl, nsites - 1);
+#define HOP_DIR(D, NEXT)                                                                      \
+  {                                                                                           \
+    if (!kPipe && (D) > 0) HOP_LOAD(__ldg(nb + (D)));                                         \
+    HOP_PROJECT(D)                                                                            \
+    const float2 sc = d.sc;                                                                   \
+    if (kPipe) { NEXT; }                                                                      \
+    dir_add<S, (D) / 2, ((D) & 1) == 0, DAG, PRE, RC, true>(acc, h, sc, lk + (D) * LC * nsites, \
+                                                            nsites);                          \
   }
+    HOP_LOAD(__ldg(nb));
+    wait_links<S>();
+    if constexpr (kPipe) {
+      HOP_DIR(0, HOP_LOAD(__ldg(nb + 1)))
+      HOP_DIR(1, HOP_LOAD(__ldg(nb + 2)))
+      HOP_DIR(2, HOP_LOAD(__ldg(nb + 3)))
+      HOP_DIR(3, HOP_LOAD(__ldg(nb + 4)))
+      HOP_DIR(4, HOP_LOAD(__ldg(nb + 5)))
+      HOP_DIR(5, HOP_LOAD(__ldg(nb + 6)))
+      HOP_DIR(6, HOP_LOAD(__ldg(nb + 7)))
+      HOP_DIR(7, )
+    } else {
+      // always taken: keeps the compiler from mixing the directions (and spilling)
+      if (P.dirs & 1) HOP_DIR(0, )
+      if (P.dirs & 2) HOP_DIR(1, )
+      if (P.dirs & 4) HOP_DIR(2, )
+      if (P.dirs & 8) HOP_DIR(3, )
+      if (P.dirs & 16) HOP_DIR(4, )
+      if (P.dirs & 32) HOP_DIR(5, )
+      if (P.dirs & 64) HOP_DIR(6, )
+      if (P.dirs & 128) HOP_DIR(7, )
+    }
+#undef HOP_DIR
+  } else {
+    // With M_phi on load every lane of the warp takes part in a direction (its
+    // halves are exchanged between lanes) and one that no lane has is skipped by
+    // all; otherwise each lane branches on its own neighbour.
+    constexpr int LC = link_words<S, RC>();
+    const size_t ls = (size_t)P.link_cs;
+    const int4 *nb = reinterpret_cast<const int4 *>(P.nbr + (size_t)(active ? site : 0) * 8);
+    const int4 lo = __ldg(nb), hi = __ldg(nb + 1);
+    const int js[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#define HOP_DIR(D)                                                                             \
+  {                                                                                            \
+    const int j = active ? js[D] : -1;                                                         \
+    const bool valid = (unsigned)j < (unsigned)P.in_limit;                                     \
+    if (PRE ? __any_sync(0xffffffffu, valid) != 0 : valid) {                                   \
+      HOP_LOAD(valid ? j : 0);                                                                 \
+      HOP_PROJECT(D)                                                                           \
+      if (valid)                                                                               \
+        dir_add<S, (D) / 2, ((D) & 1) == 0, DAG, PRE, RC, false>(                              \
+            acc, h, d.sc,                                                                      \
+            links + (size_t)((D) / 2) * LC * ls +                                              \
+                (((D) & 1) ? P.in_link_off + j : P.out_link_off + site),                       \
+            ls);                                                                               \
+    }                                                                                          \
+  }
+    HOP_DIR(0)
+    HOP_DIR(1)
+    HOP_DIR(2)
+    HOP_DIR(3)
+    HOP_DIR(4)
+    HOP_DIR(5)
+    HOP_DIR(6)
+    HOP_DIR(7)
+#undef HOP_DIR
+  }
+#undef HOP_PROJECT
+#undef HOP_LOAD
   const int e = site * Ls + s0;
   float a0[24], a1[24];
 #pragma unroll
@@ -665,53 +815,75 @@ __device__ __forceinline__ void hop2_body(const HopParams &P) {
   }
 
   if constexpr (EPI) {
+    const float p0 = cf.f.p0q, p1 = cf.f.p1q;
     if (P.inv) {
-      // y = (1 - r S)^-1 v on the lanes of the site, as a scan (no shared
-      // memory). On the components where S takes s - 1: the wrap-free
+      // z = (p0 + p1 S) y, y = (1 - r S)^-1 v, on the lanes of the site as a scan (no
+      // shared memory). On the components where S takes s - 1: the wrap-free
       // recursion yh_j = v_j + r yh_{j-1} (yh_0 = v_0) is a scan over the
-      // site's lanes with the constant factor r^2 per lane; the wrap then adds
-      // r^j d with d = -m_f r yh_{Ls-1} / (1 + m_f r^Ls) (the closed form's
-      // first element). Where S takes s + 1 the same runs in reversed order.
+      // site's lanes with the constant factor r^2 per lane (C: yh at the lane's
+      // second slice); the wrap then adds r^j d with d = -m_f r yh_{Ls-1} / (1 + m_f
+      // r^Ls) (the closed form's first element). Where S takes s + 1 the same runs
+      // in reversed order. One step of the scan runs over all 24 components, which
+      // share its factors; y at the neighbour that p1 S needs follows from the
+      // lane's own copy of C there.
       const LsK<float> &c = cf.f;
       const float r = c.r, mfr = -c.mf * c.r * c.inv_den;
-      // r^(2 jp), r^(Ls - 2 - 2 jp) and r^(2 d) for the scan steps
-      float r_lo = 1.f, r_rev = 1.f;
-      for (int i = 0; i < 2 * jp; ++i) r_lo *= r;
-      for (int i = 0; i < Ls - 2 - 2 * jp; ++i) r_rev *= r;
-      const float r2 = r * r;
-      const int base = lane - jp;
+      const int base = lane - jp, jr = np - 1 - jp;  // the lane's place in either order
+      float rd = 1.f, ru = 1.f, rl = 1.f;            // r^(2 jp), r^(2 jr), r^(Ls - 1)
+      for (int i = 0; i < 2 * jp; ++i) rd *= r;
+      for (int i = 0; i < 2 * jr; ++i) ru *= r;
+      for (int i = 0; i < Ls - 1; ++i) rl *= r;
+      float C[24];
 #pragma unroll
       for (int k = 0; k < 24; ++k) {
         const bool down = (k < 12) != DAG;
-        // order the pair along the recursion: first, second
-        const float f = down ? a0[k] : a1[k], g = down ? a1[k] : a0[k];
-        const float w1 = g + r * f;
-        float C = w1;  // inclusive scan of w1 with factor r^2 per lane step
-        float m = r2;
-        for (int d = 1; d < np; d <<= 1) {
-          const float tu = __shfl_up_sync(0xffffffffu, C, d);
-          const float td = __shfl_down_sync(0xffffffffu, C, d);
-          if (down ? (jp >= d) : (jp + d < np)) C += m * (down ? tu : td);
-          m *= m;
-        }
-        const float cu = __shfl_up_sync(0xffffffffu, C, 1);
-        const float cd = __shfl_down_sync(0xffffffffu, C, 1);
-        const float cin = down ? (jp > 0 ? cu : 0.f) : (jp + 1 < np ? cd : 0.f);
-        const float last = __shfl_sync(0xffffffffu, C, down ? base + np - 1 : base);
-        const float dl = mfr * last;
-        // positions along the recursion: first at 2 jp (down) or Ls-2-2jp
-        // counted from the other end (up), second one further
-        const float rf = down ? r_lo : r_rev, rs = rf * r;
-        const float yf = f + r * cin + rf * dl;
-        const float ys = w1 + r2 * cin + rs * dl;
-        a0[k] = down ? yf : ys;
-        a1[k] = down ? ys : yf;
+        C[k] = down ? fmaf(r, a0[k], a1[k]) : fmaf(r, a1[k], a0[k]);
       }
-    }
-    {
+      float m = r * r;
+      for (int d = 1; d < np; d <<= 1) {
+        // (selected, not multiplied by zero: the lane d away may be another site's)
+        const bool od = jp >= d, ou = jr >= d;
+#pragma unroll
+        for (int k = 0; k < 24; ++k) {
+          const bool down = (k < 12) != DAG;
+          const float t = down ? __shfl_up_sync(0xffffffffu, C[k], d)
+                               : __shfl_down_sync(0xffffffffu, C[k], d);
+          if (down ? od : ou) C[k] = fmaf(m, t, C[k]);
+        }
+        m *= m;
+      }
+      // r^(2 j - 1) at the place before the lane's first slice (the wrap: r^(Ls - 1))
+      float gd = rl, gu = rl;
+      if (jp > 0) {
+        gd = r;
+        for (int i = 0; i < 2 * jp - 2; ++i) gd *= r;
+      }
+      if (jr > 0) {
+        gu = r;
+        for (int i = 0; i < 2 * jr - 2; ++i) gu *= r;
+      }
+      const float pd = p1 * pl.fm, pu = p1 * pl.fp;
+#pragma unroll
+      for (int k = 0; k < 24; ++k) {
+        const bool down = (k < 12) != DAG;
+        const float cin = down ? __shfl_up_sync(0xffffffffu, C[k], 1)
+                               : __shfl_down_sync(0xffffffffu, C[k], 1);
+        const float last = __shfl_sync(0xffffffffu, C[k], down ? base + np - 1 : base);
+        const float dl = mfr * last;
+        const float first = down ? a0[k] : a1[k];  // v at the first slice of the order
+        const float rf = down ? rd : ru;
+        const bool inner = (down ? jp : jr) > 0;
+        const float yf = fmaf(rf, dl, fmaf(r, inner ? cin : 0.f, first));
+        const float ys = fmaf(rf * r, dl, C[k]);
+        const float before = fmaf(down ? gd : gu, dl, inner ? cin : last);
+        const float zf = fmaf(down ? pd : pu, before, p0 * yf);
+        const float zs = fmaf(p1, yf, p0 * ys);
+        a0[k] = down ? zf : zs;
+        a1[k] = down ? zs : zf;
+      }
+    } else if (p1 != 0.f) {
       // q0 (p0 + p1 S) needs only the neighbouring slices: the pair's own and
       // the outer ones from the neighbouring lanes of the site
-      const float p0 = cf.f.p0q, p1 = cf.f.p1q;
 #pragma unroll
       for (int k = 0; k < 24; ++k) {
         const bool down = (k < 12) != DAG;  // S takes s - 1 on these components
@@ -725,6 +897,12 @@ __device__ __forceinline__ void hop2_body(const HopParams &P) {
           a0[k] = p0 * t0 + p1 * t1;
           a1[k] = p0 * t1 + p1 * (pl.fp * wd);
         }
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 24; ++k) {
+        a0[k] *= p0;
+        a1[k] *= p0;
       }
     }
     // the x-term, (a0 + a1 S) x, after the Ls operator, in registers; every
@@ -756,10 +934,10 @@ __device__ __forceinline__ void hop2_body(const HopParams &P) {
   }
 }
 
-template <class S, bool DAG, bool PRE, bool RC, bool EPI>
+template <class S, bool DAG, bool PRE, bool RC, bool EPI, bool DENSE>
 __global__ void __launch_bounds__(128, 4) hop2_kernel(const __grid_constant__ HopParams P) {
   prof_enter(P);
-  hop2_body<S, DAG, PRE, RC, EPI>(P);
+  hop2_body<S, DAG, PRE, RC, EPI, DENSE>(P);
   prof_exit(P);
 }
 
@@ -780,12 +958,27 @@ int hop_sites_per_cta(int Ls, dwf_prec p) {
   return best;
 }
 
-size_t hop_smem_bytes(int Ls, dwf_prec p, int epi, int has_x) {
-  // the two-slice kernel runs its Ls epilogue across the lanes of a site
-  if (!epi || hop_pairs(Ls, p)) return 0;
+size_t hop_smem_bytes(int Ls, dwf_prec p, int epi, int has_x, int recon) {
+  // the two-slice kernel keeps the 8 links of its sites there
+  if (hop_pairs(Ls, p))
+    return (size_t)hop_sites_per_cta(Ls, p) * 8 * link_record_bytes(DWF_FP32, recon);
+  if (!epi) return 0;
   // the one-slice kernel walks the columns of T (and of x) in shared memory
   const size_t rs = (p == DWF_FP64) ? 8 : 4;
   return (size_t)hop_sites_per_cta(Ls, p) * 24 * (Ls + 1) * rs * (has_x ? 2 : 1);
+}
+
+template <class S, bool DAG, bool PRE, bool RC, bool DENSE>
+static void launch_two(const HopParams &P, dim3 grid, size_t smem, cudaStream_t st) {
+  if (P.epi) {
+    hop2_kernel<S, DAG, PRE, RC, true, DENSE><<<grid, 128, smem, st>>>(P);
+  } else {
+    if constexpr (DAG)
+      throw Error{DWF_ERR_UNSUPPORTED, "the adjoint hop always has its M_phi^+ epilogue"};
+    else
+      hop2_kernel<S, DAG, PRE, RC, false, DENSE><<<grid, 128, smem, st>>>(P);
+  }
+  DWF_CUDA_TRY(cudaGetLastError());
 }
 
 template <class S, bool DAG, bool PRE, bool RC>
@@ -795,20 +988,27 @@ static void launch_t(const HopParams &P0, int nrhs, cudaStream_t st, dwf_prec pr
   const int nsites = hop_sites_per_cta(P.Ls, prec);
   P.nsites = nsites;
   dim3 grid((P.n_out + nsites - 1) / nsites, P.nblocks, nrhs);
-  const size_t smem = hop_smem_bytes(P.Ls, prec, P.epi, P.has_x);
+  const size_t smem = hop_smem_bytes(P.Ls, prec, P.epi, P.has_x, RC ? 1 : 0);
   if (grid.x == 0) return;
   if constexpr (!std::is_same<S, F64>::value) {
     if (hop_pairs(P.Ls, prec)) {
-      dim3 block(128);
-      if (P.epi) {
-        hop2_kernel<S, DAG, PRE, RC, true><<<grid, block, smem, st>>>(P);
-      } else {
-        if constexpr (DAG)
-          throw Error{DWF_ERR_UNSUPPORTED, "the adjoint hop always has its M_phi^+ epilogue"};
-        else
-          hop2_kernel<S, DAG, PRE, RC, false><<<grid, block, smem, st>>>(P);
+      // the dense sites (whole CTAs of them), then the others
+      const int n_out = P.n_out;
+      const int nd = std::min(n_out, (P.n_dense + nsites - 1) / nsites * nsites);
+      if (nd > 0) {
+        P.n_out = nd;
+        grid.x = (nd + nsites - 1) / nsites;
+        launch_two<S, DAG, PRE, RC, true>(P, grid, smem, st);
       }
-      DWF_CUDA_TRY(cudaGetLastError());
+      if (nd < n_out) {
+        DWF_REQUIRE(nd == 0 || !P.dot, DWF_ERR_UNSUPPORTED, "a fused dot takes one launch");
+        P.n_out = n_out;
+        P.site_off = nd;
+        P.prof_again = nd > 0 ? 1 : 0;
+        if (nd > 0) P.alg_bytes = 0;
+        grid.x = (n_out - nd + nsites - 1) / nsites;
+        launch_two<S, DAG, PRE, RC, false>(P, grid, 0, st);
+      }
       return;
     }
   }
@@ -847,13 +1047,20 @@ void launch_hop(const HopParams &P, int dagger, int pre_mphi, int nrhs, cudaStre
     launch_t<S, false, false, false>(P, nrhs, st, p);
 }
 
-// Allow the one-slice hop kernels more than 48 KB of dynamic shared memory
-// (the two-slice kernels use none). Called once per device before any launch
+// Allow the hop kernels more than 48 KB of dynamic shared memory. Called once per device before any launch
 // (and so before any stream capture).
 template <class K>
 static void allow_big_smem(K *kernel) {
   DWF_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     200 * 1024));
+}
+template <class S, bool RC>
+static void prepare_two() {
+  allow_big_smem(hop2_kernel<S, false, false, RC, false, true>);
+  allow_big_smem(hop2_kernel<S, false, false, RC, true, true>);
+  allow_big_smem(hop2_kernel<S, false, true, RC, false, true>);
+  allow_big_smem(hop2_kernel<S, false, true, RC, true, true>);
+  allow_big_smem(hop2_kernel<S, true, false, RC, true, true>);
 }
 template <class S>
 static void prepare_one() {
@@ -864,6 +1071,8 @@ static void prepare_one() {
     allow_big_smem(hop_kernel<S, false, false, true>);
     allow_big_smem(hop_kernel<S, false, true, true>);
     allow_big_smem(hop_kernel<S, true, false, true>);
+    prepare_two<S, false>();
+    prepare_two<S, true>();
   }
 }
 void prepare_kernels() {

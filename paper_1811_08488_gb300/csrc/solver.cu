@@ -79,9 +79,10 @@ static HopParams global_params(const dwf_ctx *ctx, dwf_prec p, int out_parity, c
   P.links = link_ptr(ctx, p);
   P.link_cs = ctx->geo.V4;
   P.recon = (p != DWF_FP64 && ctx->act.recon12) ? 1 : 0;
-  P.nbr = ctx->nbr_dev[out_parity].as<int>();
+  P.nbr = P.nbr_read = ctx->nbr_dev[out_parity].as<int>();
   P.n_out = ctx->geo.Vh;
   P.in_limit = ctx->geo.Vh;
+  P.n_dense = ctx->geo.Vh;
   P.xown_limit = ctx->geo.Vh;
   P.out_link_off = out_parity * ctx->geo.Vh;
   P.in_link_off = (1 - out_parity) * ctx->geo.Vh;
@@ -352,6 +353,9 @@ BlockPlan *get_block_plan(dwf_ctx *ctx, const int block[4], dwf_prec inner, int 
     };
     up(bp->nbr_oe, g.nbr_oe);
     up(bp->nbr_eo, g.nbr_eo);
+    for (int sn = 0; sn < 2; ++sn)
+      for (int h = 0; h < 4; ++h)
+        if (!g.nbr_read[sn][h].empty()) up(bp->nbr_read[sn][h], g.nbr_read[sn][h]);
     up(bp->gmap_b, g.gmap_b);
     std::vector<int> own(g.gsite.size());
     const int *L = ctx->act.dims;
@@ -431,12 +435,19 @@ void block_apply_A(dwf_ctx *ctx, BlockPlan *bp, int snake, int nrhs, const doubl
   const int odd_out = snake ? g.n_o1 : g.n_ob;
   const int even_mid = snake ? g.n_e2 : g.n_b;
   const int odd_in = snake ? g.n_o1 : g.n_ob;
+  // the neighbour table of block hop h + 1 and its dense sites
+  auto sites = [&](HopParams &P, int h, const DevBuf &nbr) {
+    const DevBuf &rd = bp->nbr_read[snake ? 1 : 0][h];
+    P.n_dense = g.dense[snake ? 1 : 0][h];
+    P.nbr = nbr.as<int>();
+    P.nbr_read = rd.p ? rd.as<int>() : P.nbr;
+  };
 
   // hop 1: odd (distance <= 1) <- even block sites; u1 = K (-1/2 Dhop M_phi p)
   HopParams P = base;
   P.in = bp->fp;
   P.out = bp->fu1;
-  P.nbr = bp->nbr_oe.as<int>();
+  sites(P, 0, bp->nbr_oe);
   P.n_out = odd_out;
   P.in_limit = g.n_b;
   P.out_link_off = g.n_e2;
@@ -453,7 +464,7 @@ void block_apply_A(dwf_ctx *ctx, BlockPlan *bp, int snake, int nrhs, const doubl
   P = base;
   P.in = bp->fu1;
   P.out = bp->fy;
-  P.nbr = bp->nbr_eo.as<int>();
+  sites(P, 1, bp->nbr_eo);
   P.n_out = even_mid;
   P.in_limit = odd_in;
   P.out_link_off = 0;
@@ -484,7 +495,7 @@ void block_apply_A(dwf_ctx *ctx, BlockPlan *bp, int snake, int nrhs, const doubl
   P = base;
   P.in = schur ? bp->fw2 : bp->fy;
   P.out = bp->fu2;
-  P.nbr = bp->nbr_oe.as<int>();
+  sites(P, 2, bp->nbr_oe);
   P.n_out = odd_out;
   P.in_limit = even_mid;
   P.out_link_off = g.n_e2;
@@ -498,7 +509,7 @@ void block_apply_A(dwf_ctx *ctx, BlockPlan *bp, int snake, int nrhs, const doubl
   P = base;
   P.in = bp->fu2;
   P.out = bp->fAp;
-  P.nbr = bp->nbr_eo.as<int>();
+  sites(P, 3, bp->nbr_eo);
   P.n_out = g.n_b;
   P.in_limit = odd_in;
   P.out_link_off = 0;

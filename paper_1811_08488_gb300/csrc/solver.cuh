@@ -52,6 +52,7 @@ struct BlockPlan {
   int nrhs = 0;
   int Ls = 0;
   DevBuf nbr_oe, nbr_eo, gmap_b, gowner;
+  DevBuf nbr_read[2][4];  // BlockGeometry::nbr_read
   DevBuf links;
   long long link_bstride = 0;
   DevBuf r, p, Ap, x, u1, y, u2, w2;
