@@ -120,18 +120,123 @@ __global__ void export_kernel(C *canon, const char *native, long long nstride, l
   }
 }
 
+// The same through shared memory. An element's 24 reals are contiguous in the
+// canonical field, where h runs fastest, and its chunks run with s fastest in the
+// native one: a thread per element touches 192-byte pieces nsite * 192 bytes apart
+// on one side. A CTA takes kIoElems / Ls sites with all their slices: the canonical
+// side moves as [s][sites], 16 bytes per thread and contiguous over the sites, the
+// native side as one element per thread; rows of the tile are padded by 16 bytes so
+// that neighbouring s fall on different banks. HBM-bound: a field of 24^3 x 64 x 16
+// (complex128 in, FP32 native, and back; 4.1 GB) 2750 us the direct way, 627 us
+// this way (6.5 TB/s).
+constexpr int kIoElems = 128;
+template <class C> __host__ __device__ inline int io_row(int sites) {  // bytes of one s
+  return sites * 24 * (int)sizeof(C) + 16;
+}
+template <class S, class C>
+__global__ void __launch_bounds__(kIoElems) import_tile_kernel(char *native, long long nstride,
+                                                               long long soff, const C *canon,
+                                                               int nsite, int Ls, int sites) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int rhs = blockIdx.y, h0 = blockIdx.x * sites, nh = min(sites, nsite - h0);
+  const int row = io_row<C>(sites), words = nh * 24 * (int)sizeof(C) / 16;
+  for (int s = 0; s < Ls; ++s) {
+    const uint4 *src = reinterpret_cast<const uint4 *>(
+        canon + (((size_t)rhs * Ls + s) * nsite + h0) * 24);
+    for (int w = threadIdx.x; w < words; w += kIoElems)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                       static_cast<uint32_t>(__cvta_generic_to_shared(smem_raw + s * row + w * 16))),
+                   "l"(src + w)
+                   : "memory");
+  }
+  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  for (int e = threadIdx.x; e < nh * Ls; e += kIoElems) {
+    const int h = e / Ls, s = e - h * Ls;
+    const C *src = reinterpret_cast<const C *>(smem_raw + s * row) + h * 24;
+    typename S::R v[24];
+    constexpr int kPer = 16 / sizeof(C);
+#pragma unroll
+    for (int k = 0; k < 24; k += kPer) {
+      const uint4 q = *reinterpret_cast<const uint4 *>(src + k);
+      C c[kPer];
+      memcpy(c, &q, 16);
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) v[k + i] = (typename S::R)c[i];
+    }
+    store24<S>(native + rhs * nstride, soff, nsite * Ls, h0 * Ls + e, v);
+  }
+}
+
+template <class S, class C>
+__global__ void __launch_bounds__(kIoElems) export_tile_kernel(C *canon, const char *native,
+                                                               long long nstride, long long soff,
+                                                               int nsite, int Ls, int sites) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int rhs = blockIdx.y, h0 = blockIdx.x * sites, nh = min(sites, nsite - h0);
+  const int row = io_row<C>(sites), words = nh * 24 * (int)sizeof(C) / 16;
+  for (int e = threadIdx.x; e < nh * Ls; e += kIoElems) {
+    const int h = e / Ls, s = e - h * Ls;
+    C *dst = reinterpret_cast<C *>(smem_raw + s * row) + h * 24;
+    typename S::R v[24];
+    load24<S>(native + rhs * nstride, soff, nsite * Ls, h0 * Ls + e, v);
+    constexpr int kPer = 16 / sizeof(C);
+#pragma unroll
+    for (int k = 0; k < 24; k += kPer) {
+      C c[kPer];
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) c[i] = (C)v[k + i];
+      uint4 q;
+      memcpy(&q, c, 16);
+      *reinterpret_cast<uint4 *>(dst + k) = q;
+    }
+  }
+  __syncthreads();
+  for (int s = 0; s < Ls; ++s) {
+    uint4 *dst = reinterpret_cast<uint4 *>(canon + (((size_t)rhs * Ls + s) * nsite + h0) * 24);
+    for (int w = threadIdx.x; w < words; w += kIoElems)
+      dst[w] = *reinterpret_cast<const uint4 *>(smem_raw + s * row + w * 16);
+  }
+}
+
+// The tile kernels move 16 bytes at a time: the canonical field has to start on a
+// 16-byte boundary (every row of sites then does). Others take the direct kernels.
+static bool io_tiled(const void *canon) { return reinterpret_cast<uintptr_t>(canon) % 16 == 0; }
+
+template <class S, class C>
+static void import_go(char *native, long long nstride, long long soff, const C *canon, int nsite,
+                      int Ls, int nrhs, cudaStream_t st) {
+  if (io_tiled(canon)) {
+    const int sites = std::max(1, kIoElems / Ls);
+    import_tile_kernel<S, C><<<dim3((nsite + sites - 1) / sites, nrhs), kIoElems,
+                               (size_t)Ls * io_row<C>(sites), st>>>(native, nstride, soff, canon,
+                                                                    nsite, Ls, sites);
+  } else {
+    import_kernel<S, C><<<dim3(1024, nrhs), 256, 0, st>>>(native, nstride, soff, canon, nsite, Ls);
+  }
+}
+template <class S, class C>
+static void export_go(C *canon, const char *native, long long nstride, long long soff, int nsite,
+                      int Ls, int nrhs, cudaStream_t st) {
+  if (io_tiled(canon)) {
+    const int sites = std::max(1, kIoElems / Ls);
+    export_tile_kernel<S, C><<<dim3((nsite + sites - 1) / sites, nrhs), kIoElems,
+                               (size_t)Ls * io_row<C>(sites), st>>>(canon, native, nstride, soff,
+                                                                    nsite, Ls, sites);
+  } else {
+    export_kernel<S, C><<<dim3(1024, nrhs), 256, 0, st>>>(canon, native, nstride, soff, nsite, Ls);
+  }
+}
+
 void launch_import(dwf_prec p, char *native, long long nstride, const void *canon, int canon_fp32,
                    int nsite, int Ls, const int *, int nrhs, cudaStream_t st) {
   const long long soff = (long long)align_up(field_data_bytes(p, nsite, Ls), 256);
-  dim3 grid(1024, nrhs), block(256);
-#define IMP(ST)                                                                          \
-  do {                                                                                   \
-    if (canon_fp32)                                                                      \
-      import_kernel<ST, float><<<grid, block, 0, st>>>(native, nstride, soff,            \
-                                                       (const float *)canon, nsite, Ls); \
-    else                                                                                 \
-      import_kernel<ST, double><<<grid, block, 0, st>>>(native, nstride, soff,           \
-                                                        (const double *)canon, nsite, Ls); \
+#define IMP(ST)                                                                             \
+  do {                                                                                      \
+    if (canon_fp32)                                                                         \
+      import_go<ST>(native, nstride, soff, (const float *)canon, nsite, Ls, nrhs, st);      \
+    else                                                                                    \
+      import_go<ST>(native, nstride, soff, (const double *)canon, nsite, Ls, nrhs, st);     \
   } while (0)
   switch (p) {
     case DWF_FP64: IMP(F64); break;
@@ -146,15 +251,12 @@ void launch_import(dwf_prec p, char *native, long long nstride, const void *cano
 void launch_export(dwf_prec p, void *canon, int canon_fp32, const char *native, long long nstride,
                    int nsite, int Ls, const int *, int nrhs, cudaStream_t st) {
   const long long soff = (long long)align_up(field_data_bytes(p, nsite, Ls), 256);
-  dim3 grid(1024, nrhs), block(256);
-#define EXP(ST)                                                                               \
-  do {                                                                                        \
-    if (canon_fp32)                                                                           \
-      export_kernel<ST, float><<<grid, block, 0, st>>>((float *)canon, native, nstride, soff, \
-                                                       nsite, Ls);                            \
-    else                                                                                      \
-      export_kernel<ST, double><<<grid, block, 0, st>>>((double *)canon, native, nstride,     \
-                                                        soff, nsite, Ls);                     \
+#define EXP(ST)                                                                             \
+  do {                                                                                      \
+    if (canon_fp32)                                                                         \
+      export_go<ST>((float *)canon, native, nstride, soff, nsite, Ls, nrhs, st);            \
+    else                                                                                    \
+      export_go<ST>((double *)canon, native, nstride, soff, nsite, Ls, nrhs, st);           \
   } while (0)
   switch (p) {
     case DWF_FP64: EXP(F64); break;
