@@ -33,7 +33,7 @@ constexpr int kEigThreads = 256;
 constexpr int kEigCtas = 152 * 4;  // CTAs of one vector-kernel launch over all its tiles
 constexpr int kMaxTiles = (kMaxEig / 4) * (kMaxEig / 4);
 
-constexpr int kMaxValues = 128;  // partial sums per CTA of one multi-dot launch at most
+constexpr int kMaxValues = 256;  // partial sums per CTA of one multi-dot launch at most
 
 size_t dot_scratch_bytes() {
   // partials: at most max(kEigCtas, kMaxTiles) CTAs x kMaxValues values;
@@ -69,6 +69,18 @@ static int wave_ctas() {
   DWF_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, K, kEigThreads, 0));
   const int n = std::max(1, per) * std::max(1, nsm);
   if (slot) slot->store(n, std::memory_order_relaxed);
+  return n;
+}
+
+// SMs of the current device.
+static int sm_count() {
+  constexpr int kDevices = 64;
+  static std::atomic<int> cache[kDevices];  // 0 until read
+  int dev = 0, n = 0;
+  DWF_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < kDevices && (n = cache[dev].load(std::memory_order_relaxed)) > 0) return n;
+  DWF_CUDA_TRY(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+  if (dev < kDevices) cache[dev].store(n, std::memory_order_relaxed);
   return n;
 }
 
@@ -196,7 +208,7 @@ __global__ void __launch_bounds__(kEigThreads) gram_kernel(const GramArgs a) {
   if (threadIdx.x == 0) a.counters[tile] = 0u;
 }
 
-// Few Y vectors (ny <= NJ <= 4) against many X (FP32, or FP16 with scales):
+// Few Y vectors (ny <= NJ <= 4) against many X, one of them not FP32:
 // the 8 warps of a CTA walk the same stretch of 32 elements (groups of 4 reals
 // or 16-byte chunks of 8 reals), warp w taking X vectors
 // ibase + w + 8 t (t < NI) and every Y vector, so each X vector is read once
@@ -313,6 +325,155 @@ __global__ void __launch_bounds__(kEigThreads) gram_skinny_kernel(const GramArgs
   if (threadIdx.x == 0) a.counters[tile] = 0u;
 }
 
+// FP32 X against few FP32 Y (ny <= NJ): the fields are flat arrays, so the CTA streams
+// segments of 64 float4 of 8 NI vectors X and of every Y through a ring of stages in
+// shared memory (cp.async, kStreamBytes of them in flight per CTA), and warp w
+// takes the X vectors ibase + w + 8 t against every Y from there. 24 X and 4 Y on
+// 16^3 x 32 x 12 (2.1 GB): 458 us, bound by issue (56%) and its barriers, against
+// 823 us with loads into registers, a dozen per thread in flight, which waited two
+// thirds of the time. Two complex
+// products at a time are added in FP32 as (re, im) pairs, then compensated.
+constexpr int kSeg = 64;  // float4 of one vector in a stage
+constexpr int kStreamBytes = 110 * 1024;
+template <int NI, int NJ> constexpr int stream_stages() {
+  constexpr int n = kStreamBytes / ((8 * NI + NJ) * kSeg * 16);
+  return n < 2 ? 2 : n > 6 ? 6 : n;
+}
+
+template <int NI, int NJ>
+__global__ void __launch_bounds__(kEigThreads, 2) gram_stream_kernel(const GramArgs a) {
+  constexpr int NV = 8 * NI * NJ * 2, NVEC = 8 * NI + NJ, kStages = stream_stages<NI, NJ>();
+  static_assert(NV <= kMaxValues, "too many partial sums per CTA");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int s_last;
+  float4 *ring = reinterpret_cast<float4 *>(smem_raw);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int tile = blockIdx.y, ibase = tile * 8 * NI;
+  const long long nseg = (a.n4 + kSeg - 1) / kSeg;
+  // thread t copies float4 t % 64 of the X vectors ibase + t / 64 + 4 m and of Y t / 64
+  const int v0 = threadIdx.x / kSeg, off = threadIdx.x % kSeg;
+  const char *xp = a.x + (ibase + v0) * a.xvs + off * 16, *yp = a.y + v0 * a.yvs + off * 16;
+  const int xn = a.nx - ibase - v0;  // vector 4 m is there if 4 m < xn
+  const uint32_t dst0 = static_cast<uint32_t>(__cvta_generic_to_shared(ring + threadIdx.x));
+  auto load = [&](long long seg, int stage) {
+    if (seg < nseg) {
+      const bool in = seg * kSeg + off < a.n4;
+      const uint32_t dst = dst0 + stage * (NVEC * kSeg * 16);
+      auto copy = [&](uint32_t to, const char *src, bool ok) {
+        const int bytes = ok ? 16 : 0;  // 0: filled with zeros
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to),
+                     "l"(ok ? src : a.x), "r"(bytes)
+                     : "memory");
+      };
+      const char *x = xp + seg * (kSeg * 16);
+#pragma unroll
+      for (int m = 0; m < 2 * NI; ++m)
+        copy(dst + m * (4 * kSeg * 16), x + m * 4 * a.xvs, in && 4 * m < xn);
+      if (v0 < NJ)
+        copy(dst + 2 * NI * (4 * kSeg * 16), yp + seg * (kSeg * 16), in && v0 < a.ny);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  KahanF acc[NI][NJ][2];
+  for (int q = 0; q < kStages - 1; ++q) load(blockIdx.x + (long long)q * gridDim.x, q);
+  int stage = 0;
+  for (long long seg = blockIdx.x; seg < nseg; seg += gridDim.x) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+    __syncthreads();  // this stage has arrived, and the one before it has been read
+    load(seg + (long long)(kStages - 1) * gridDim.x, stage == 0 ? kStages - 1 : stage - 1);
+    const float4 *st = ring + stage * NVEC * kSeg;
+    float y[NJ][8];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const float4 p = st[(8 * NI + j) * kSeg + lane], q = st[(8 * NI + j) * kSeg + 32 + lane];
+      y[j][0] = p.x; y[j][1] = p.y; y[j][2] = p.z; y[j][3] = p.w;
+      y[j][4] = q.x; y[j][5] = q.y; y[j][6] = q.z; y[j][7] = q.w;
+    }
+#pragma unroll
+    for (int t = 0; t < NI; ++t) {
+      const float4 p = st[(w + 8 * t) * kSeg + lane], q = st[(w + 8 * t) * kSeg + 32 + lane];
+      const float x[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        // conj(x) y: (re, im) = x_re (y_re, y_im) + x_im (y_im, -y_re), two complex
+        // products at a time
+#pragma unroll
+        for (int g = 0; g < 8; g += 4) {
+          float2 d = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int k = g; k < g + 4; k += 2) {
+            d = __ffma2_rn(make_float2(x[k], x[k]), make_float2(y[j][k], y[j][k + 1]), d);
+            d = __ffma2_rn(make_float2(x[k + 1], x[k + 1]), make_float2(y[j][k + 1], -y[j][k]), d);
+          }
+          acc[t][j][0].add(d.x);
+          acc[t][j][1].add(d.y);
+        }
+      }
+    }
+    stage = stage + 1 == kStages ? 0 : stage + 1;
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  // value v = ((w NI + t) NJ + j) 2 + c: warp sums, written by lane 0 of warp w
+  double *part = a.partials + (size_t)tile * gridDim.x * NV;
+#pragma unroll
+  for (int t = 0; t < NI; ++t)
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        double d = acc[t][j][c].value();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+        if (lane == 0)
+          part[(size_t)(((w * NI + t) * NJ + j) * 2 + c) * gridDim.x + blockIdx.x] = d;
+      }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned int prev = atomicAdd(a.counters + tile, 1u);
+    s_last = prev == gridDim.x - 1u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  // the last CTA: a warp per value, in a fixed order
+  for (int v = w; v < NV; v += kEigThreads / 32) {
+    const volatile double *vp = part + (size_t)v * gridDim.x;
+    double sum = 0.0;
+    for (unsigned int k = lane; k < gridDim.x; k += 32) sum += vp[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+    const int c = v & 1, j = (v >> 1) % NJ, wt = (v >> 1) / NJ;
+    const int gi = ibase + wt / NI + 8 * (wt % NI);
+    if (lane == 0 && gi < a.nx && j < a.ny)
+      reinterpret_cast<double *>(a.G + (size_t)gi * a.ldg + j)[c] = sum;
+  }
+  if (threadIdx.x == 0) a.counters[tile] = 0u;
+}
+
+template <int NI, int NJ>
+static void gram_stream_go(const GramArgs &a, cudaStream_t st) {
+  constexpr int bytes = stream_stages<NI, NJ>() * (8 * NI + NJ) * kSeg * 16;
+  DWF_CUDA_TRY(cudaFuncSetAttribute(gram_stream_kernel<NI, NJ>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  const int tiles = (a.nx + 8 * NI - 1) / (8 * NI);
+  const dim3 grid(ctas_per_tile(2 * sm_count(), tiles, a.n4, kSeg), tiles);
+  gram_stream_kernel<NI, NJ><<<grid, kEigThreads, bytes, st>>>(a);
+  DWF_CUDA_TRY(cudaGetLastError());
+}
+// All X in one tile of up to 32 vectors, so that the Y are read once.
+template <int NJ>
+static void gram_stream(const GramArgs &a, cudaStream_t st) {
+  if (a.nx <= 8)
+    gram_stream_go<1, NJ>(a, st);
+  else if (a.nx <= 16)
+    gram_stream_go<2, NJ>(a, st);
+  else if (a.nx <= 24)
+    gram_stream_go<3, NJ>(a, st);
+  else
+    gram_stream_go<4, NJ>(a, st);
+}
+
 template <int NI, int NJ, class SX, class SY>
 static void gram_skinny_go(const GramArgs &a, cudaStream_t st) {
   const int tiles = (a.nx + 8 * NI - 1) / (8 * NI);
@@ -328,8 +489,7 @@ static void gram_skinny_launch(const GramArgs &a, dwf_prec xprec, dwf_prec yprec
     yprec == DWF_FP64 ? gram_skinny_go<NI, NJ, F16, F64>(a, st)
                       : gram_skinny_go<NI, NJ, F16, F32>(a, st);
   else
-    yprec == DWF_FP64 ? gram_skinny_go<NI, NJ, F32, F64>(a, st)
-                      : gram_skinny_go<NI, NJ, F32, F32>(a, st);
+    gram_skinny_go<NI, NJ, F32, F64>(a, st);  // (FP32 Y: gram_stream)
 }
 
 template <int TI, int TJ>
@@ -369,7 +529,14 @@ void gram(const VecSet &X, const VecSet &Y, long long cs, double2 *G, int ldg,
   a.ldg = ldg;
   a.partials = w.partials;
   a.counters = w.counters;
-  if (Y.n == 1)
+  if (Y.n <= 4 && X.prec == DWF_FP32 && Y.prec == DWF_FP32) {
+    if (Y.n == 1)
+      gram_stream<1>(a, st);
+    else if (Y.n == 2)
+      gram_stream<2>(a, st);
+    else
+      gram_stream<4>(a, st);
+  } else if (Y.n == 1)
     gram_skinny_launch<2, 1>(a, X.prec, Y.prec, st);
   else if (Y.n == 2)
     gram_skinny_launch<2, 2>(a, X.prec, Y.prec, st);
