@@ -173,14 +173,38 @@ def _ptr(t) -> int:
     return t.data_ptr() if hasattr(t, "data_ptr") else int(t)
 
 
+_current_stream = None  # torch.cuda.current_stream, once torch is needed
+
+
 def _stream(stream):
+    global _current_stream
     if stream is not None:
-        return C.c_void_p(stream)
-    import torch
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return stream
+    if _current_stream is None:
+        import torch
+        _current_stream = torch.cuda.current_stream
+    return _current_stream().cuda_stream
+
+
+class _MassList:
+    """Masses given as a list: an array of C doubles and its length."""
+    __slots__ = ("size", "arr")
+
+    def __init__(self, mf):
+        self.size = len(mf)
+        self.arr = (C.c_double * self.size)(*mf)
+
+    def __iter__(self):
+        return iter(self.arr)
 
 
 def _masses(mf, nrhs=None):
+    """(masses with .size, pointer). A list of floats, the usual argument of the
+    operator calls, is copied straight to C doubles: through numpy the pointer alone
+    took longer than the smallest hop."""
+    if type(mf) is list and nrhs is None and mf and all(type(v) is float for v in mf):
+        m = _MassList(mf)
+        return m, m.arr
     m = np.atleast_1d(np.asarray(mf, dtype=np.float64))
     if nrhs is not None and m.size == 1 and nrhs > 1:
         m = np.repeat(m, nrhs)
@@ -248,102 +272,102 @@ class Context:
 
     def field_import(self, native, prec, canon, nrhs=1, stream=None):
         fp32 = int(str(canon.dtype).endswith("complex64"))
-        self._check(lib().dwf_field_import(self._h, C.c_void_p(_ptr(native)), PREC.get(prec, prec),
-                                           C.c_void_p(_ptr(canon)), fp32, nrhs, _stream(stream)))
+        self._check(lib().dwf_field_import(self._h, _ptr(native), PREC.get(prec, prec),
+                                           _ptr(canon), fp32, nrhs, _stream(stream)))
 
     def field_export(self, canon, native, prec, nrhs=1, stream=None):
         fp32 = int(str(canon.dtype).endswith("complex64"))
-        self._check(lib().dwf_field_export(self._h, C.c_void_p(_ptr(canon)), fp32,
-                                           C.c_void_p(_ptr(native)), PREC.get(prec, prec), nrhs,
+        self._check(lib().dwf_field_export(self._h, _ptr(canon), fp32,
+                                           _ptr(native), PREC.get(prec, prec), nrhs,
                                            _stream(stream)))
 
     # --------------------------------------------------------------- operators
     def dslash_eo(self, out, inp, out_parity, dagger, prec, mf, stream=None):
         m, mp = _masses(mf)
-        self._check(lib().dwf_dslash_eo(self._h, C.c_void_p(_ptr(out)), C.c_void_p(_ptr(inp)),
+        self._check(lib().dwf_dslash_eo(self._h, _ptr(out), _ptr(inp),
                                         out_parity, int(dagger), PREC.get(prec, prec), m.size, mp,
                                         _stream(stream)))
 
     def m5(self, out, inp, dagger, prec, mf, stream=None):
         m, mp = _masses(mf)
-        self._check(lib().dwf_m5(self._h, C.c_void_p(_ptr(out)), C.c_void_p(_ptr(inp)), int(dagger),
+        self._check(lib().dwf_m5(self._h, _ptr(out), _ptr(inp), int(dagger),
                                  PREC.get(prec, prec), m.size, mp, _stream(stream)))
 
     def m5inv(self, out, inp, dagger, prec, mf, stream=None):
         m, mp = _masses(mf)
-        self._check(lib().dwf_m5inv(self._h, C.c_void_p(_ptr(out)), C.c_void_p(_ptr(inp)),
+        self._check(lib().dwf_m5inv(self._h, _ptr(out), _ptr(inp),
                                     int(dagger), PREC.get(prec, prec), m.size, mp, _stream(stream)))
 
     def m5inv_gemm(self, out, inp, dagger, prec, mf, stream=None):
         """dwf_m5inv_gemm: M_5^-1 (dagger: its adjoint) on the tensor cores,
         all right-hand sides of `mf` in one launch."""
         m, mp = _masses(mf)
-        self._check(lib().dwf_m5inv_gemm(self._h, C.c_void_p(_ptr(out)), C.c_void_p(_ptr(inp)),
+        self._check(lib().dwf_m5inv_gemm(self._h, _ptr(out), _ptr(inp),
                                          int(dagger), PREC.get(prec, prec), m.size, mp,
                                          _stream(stream)))
 
     def mpc(self, out, inp, dagger, prec, mf, stream=None):
         m, mp = _masses(mf)
-        self._check(lib().dwf_mpc(self._h, C.c_void_p(_ptr(out)), C.c_void_p(_ptr(inp)), int(dagger),
+        self._check(lib().dwf_mpc(self._h, _ptr(out), _ptr(inp), int(dagger),
                                   PREC.get(prec, prec), m.size, mp, _stream(stream)))
 
     def mpc_sym(self, out, inp, dagger, prec, mf, stream=None):
         """dwf_mpc_sym: D_sym = 1 - M_5^-1 M^4_eo M_5^-1 M^4_oe (or its adjoint)."""
         m, mp = _masses(mf)
-        self._check(lib().dwf_mpc_sym(self._h, C.c_void_p(_ptr(out)), C.c_void_p(_ptr(inp)),
+        self._check(lib().dwf_mpc_sym(self._h, _ptr(out), _ptr(inp),
                                       int(dagger), PREC.get(prec, prec), m.size, mp,
                                       _stream(stream)))
 
     def mdagm_sym(self, out, inp, prec, mf, stream=None):
         """dwf_mdagm_sym: D_sym^+ D_sym."""
         m, mp = _masses(mf)
-        self._check(lib().dwf_mdagm_sym(self._h, C.c_void_p(_ptr(out)), C.c_void_p(_ptr(inp)),
+        self._check(lib().dwf_mdagm_sym(self._h, _ptr(out), _ptr(inp),
                                         PREC.get(prec, prec), m.size, mp, _stream(stream)))
 
     def mdagm(self, out, inp, prec, mf, stream=None):
         m, mp = _masses(mf)
-        self._check(lib().dwf_mdagm(self._h, C.c_void_p(_ptr(out)), C.c_void_p(_ptr(inp)),
+        self._check(lib().dwf_mdagm(self._h, _ptr(out), _ptr(inp),
                                     PREC.get(prec, prec), m.size, mp, _stream(stream)))
 
     def mdagm_noalloc(self, out, inp, prec, mf, stream=None):
         """D_PC^+ D_PC without device allocation (temporaries in the library's
         fixed scratch array of NOALLOC_SCRATCH_BYTES)."""
         m, mp = _masses(mf)
-        self._check(lib().dwf_mdagm_noalloc(self._h, C.c_void_p(_ptr(out)), C.c_void_p(_ptr(inp)),
+        self._check(lib().dwf_mdagm_noalloc(self._h, _ptr(out), _ptr(inp),
                                             PREC.get(prec, prec), m.size, mp, _stream(stream)))
 
     def block_apply(self, out, inp, params, mf, stream=None):
         m, mp = _masses(mf)
-        self._check(lib().dwf_block_apply(self._h, C.c_void_p(_ptr(out)), C.c_void_p(_ptr(inp)),
+        self._check(lib().dwf_block_apply(self._h, _ptr(out), _ptr(inp),
                                           C.byref(params), m.size, mp, _stream(stream)))
 
     def block_precond(self, z, r, params, mf, stream=None):
         m, mp = _masses(mf)
-        self._check(lib().dwf_block_precond(self._h, C.c_void_p(_ptr(z)), C.c_void_p(_ptr(r)),
+        self._check(lib().dwf_block_precond(self._h, _ptr(z), _ptr(r),
                                             C.byref(params), m.size, mp, _stream(stream)))
 
     # ------------------------------------------------------------------- solve
     def source_prep(self, b_even, phi_even, phi_odd, prec, mf, stream=None):
         """dwf_source_prep: b = D_PC^+ (phi_e - M^4_eo M_5^-1 phi_o), native fields."""
         m, mp = _masses(mf)
-        self._check(lib().dwf_source_prep(self._h, C.c_void_p(_ptr(b_even)),
-                                          C.c_void_p(_ptr(phi_even)), C.c_void_p(_ptr(phi_odd)),
+        self._check(lib().dwf_source_prep(self._h, _ptr(b_even),
+                                          _ptr(phi_even), _ptr(phi_odd),
                                           PREC.get(prec, prec), m.size, mp, _stream(stream)))
 
     def source_prep_sym(self, b_even, phi_even, phi_odd, prec, mf, stream=None):
         """dwf_source_prep_sym: b = D_sym^+ M_5^-1 (phi_e - M^4_eo M_5^-1 phi_o)."""
         m, mp = _masses(mf)
-        self._check(lib().dwf_source_prep_sym(self._h, C.c_void_p(_ptr(b_even)),
-                                              C.c_void_p(_ptr(phi_even)),
-                                              C.c_void_p(_ptr(phi_odd)), PREC.get(prec, prec),
+        self._check(lib().dwf_source_prep_sym(self._h, _ptr(b_even),
+                                              _ptr(phi_even),
+                                              _ptr(phi_odd), PREC.get(prec, prec),
                                               m.size, mp, _stream(stream)))
 
     def odd_reconstruct(self, psi_odd, psi_even, phi_odd, prec, mf, stream=None):
         """dwf_odd_reconstruct: psi_o = M_5^-1 (phi_o - M^4_oe psi_e), native fields."""
         m, mp = _masses(mf)
-        self._check(lib().dwf_odd_reconstruct(self._h, C.c_void_p(_ptr(psi_odd)),
-                                              C.c_void_p(_ptr(psi_even)),
-                                              C.c_void_p(_ptr(phi_odd)), PREC.get(prec, prec),
+        self._check(lib().dwf_odd_reconstruct(self._h, _ptr(psi_odd),
+                                              _ptr(psi_even),
+                                              _ptr(phi_odd), PREC.get(prec, prec),
                                               m.size, mp, _stream(stream)))
 
     def solve_full(self, phi_even, phi_odd, mf, params, stream=None):
@@ -413,7 +437,7 @@ class Context:
         theta = np.zeros(m)
         resid = np.zeros(m)
         info = EigInfo()
-        self._check(lib().dwf_eig_lowmodes(self._h, C.c_void_p(_ptr(V)), int(m), float(mf),
+        self._check(lib().dwf_eig_lowmodes(self._h, _ptr(V), int(m), float(mf),
                                            C.byref(params),
                                            theta.ctypes.data_as(C.POINTER(C.c_double)),
                                            resid.ctypes.data_as(C.POINTER(C.c_double)),
@@ -422,16 +446,16 @@ class Context:
 
     def field_convert(self, out, out_prec, inp, in_prec, nrhs=1, stream=None):
         """dwf_field_convert: native fields from in_prec to out_prec."""
-        self._check(lib().dwf_field_convert(self._h, C.c_void_p(_ptr(out)),
-                                            PREC.get(out_prec, out_prec), C.c_void_p(_ptr(inp)),
+        self._check(lib().dwf_field_convert(self._h, _ptr(out),
+                                            PREC.get(out_prec, out_prec), _ptr(inp),
                                             PREC.get(in_prec, in_prec), int(nrhs),
                                             _stream(stream)))
 
     def deflate(self, z, r, V, lam, prec, nrhs=1, accumulate=False, vprec="fp32", stream=None):
         """dwf_deflate: z = (z if accumulate) + V Lambda^-1 V^+ r."""
         lam = np.ascontiguousarray(lam, dtype=np.float64)
-        self._check(lib().dwf_deflate(self._h, C.c_void_p(_ptr(z)), C.c_void_p(_ptr(r)),
-                                      C.c_void_p(_ptr(V)), PREC.get(vprec, vprec),
+        self._check(lib().dwf_deflate(self._h, _ptr(z), _ptr(r),
+                                      _ptr(V), PREC.get(vprec, vprec),
                                       lam.ctypes.data_as(C.POINTER(C.c_double)), lam.size,
                                       PREC.get(prec, prec), int(nrhs), int(bool(accumulate)),
                                       _stream(stream)))
@@ -446,7 +470,7 @@ class Context:
         xp = x.ctypes.data if isinstance(x, np.ndarray) else _ptr(x)
         bp = b.ctypes.data if isinstance(b, np.ndarray) else _ptr(b)
         st = lib().mspcg_solve_deflated(self._h, C.c_void_p(xp), C.c_void_p(bp), m.size, mp,
-                                        C.byref(params), C.c_void_p(_ptr(V)),
+                                        C.byref(params), _ptr(V),
                                         PREC.get(vprec, vprec),
                                         lam.ctypes.data_as(C.POINTER(C.c_double)), lam.size,
                                         int(bool(coarse)), infos, _stream(stream))
