@@ -66,6 +66,7 @@ KNOWN_TRAFFIC = {
     "hop2_kernel<F16,1,0,0,1> [block]": {"bytes": 1799313536, "source_sha": "a5428b9e50878f1d"},
 }
 HOP_SOURCES = ["paper_1811_08488_gb300/csrc/hop.cu", "paper_1811_08488_gb300/csrc/device_common.cuh",
+               "paper_1811_08488_gb300/csrc/ls_lanes.cuh",
                "paper_1811_08488_gb300/csrc/dwf_internal.cuh"]
 
 

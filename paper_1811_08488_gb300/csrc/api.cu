@@ -431,7 +431,7 @@ dwf_status dwf_block_apply(dwf_ctx *ctx, void *out, const void *in,
   DWF_REQUIRE(out && in && out != in, DWF_ERR_INVALID_ARG, "null or aliased fields");
   DWF_REQUIRE(ctx->have_gauge, DWF_ERR_NO_GAUGE, "no gauge field loaded");
   cudaStream_t st = (cudaStream_t)stream;
-  dwf::BlockPlan *bp = dwf::get_block_plan(ctx, params->block, params->inner, nrhs, st);
+  dwf::BlockPlan *bp = dwf::get_block_plan(ctx, params->block, params->inner, nrhs, params->snake, st);
   dwf::BlockArgs B = dwf::block_args(ctx, bp, (char *)out, (const char *)in, nullptr, 0, nullptr);
   dwf::block_gather(bp->inner, B, nrhs, st);
   dwf::block_apply_A(ctx, bp, params->snake, nrhs, mf, false, nullptr, st, params->schur);
@@ -449,7 +449,7 @@ dwf_status dwf_block_precond(dwf_ctx *ctx, void *z, const void *r,
   DWF_REQUIRE(params->inner_iters >= 1, DWF_ERR_INVALID_ARG, "inner_iters must be >= 1");
   DWF_REQUIRE(ctx->have_gauge, DWF_ERR_NO_GAUGE, "no gauge field loaded");
   cudaStream_t st = (cudaStream_t)stream;
-  dwf::BlockPlan *bp = dwf::get_block_plan(ctx, params->block, params->inner, nrhs, st);
+  dwf::BlockPlan *bp = dwf::get_block_plan(ctx, params->block, params->inner, nrhs, params->snake, st);
   dwf::block_precondition(ctx, bp, (char *)z, (const char *)r, params->inner_iters,
                           params->snake, nrhs, mf, nullptr, 0, nullptr, st, DWF_FP32, nullptr,
                           nullptr, params->inner_tol, params->schur);

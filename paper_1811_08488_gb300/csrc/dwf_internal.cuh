@@ -206,6 +206,7 @@ struct BlockGeometry {
   std::vector<int> gsite;   // [nblocks][n_comb] global lexicographic site of each owner
   // leading sites of each block hop with all or most neighbours [snake][hop 1..4], and
   // their neighbours with the absent ones replaced (empty where none is absent)
+  // (filled by find_dense_sites)
   int dense[2][4];
   std::vector<int> nbr_read[2][4];
   std::vector<int> gmap_b;  // [nblocks][n_b] global even half index of block sites
@@ -213,6 +214,7 @@ struct BlockGeometry {
 
 void build_geometry(Geometry &g, const int dims[4]);
 void build_block_geometry(BlockGeometry &bg, const int dims[4], const int block[4]);
+void find_dense_sites(BlockGeometry &bg, int snake);
 
 // ---------------------------------------------------------------------------
 // Device buffers

@@ -183,15 +183,6 @@ void build_block_geometry(BlockGeometry &bg, const int dims[4], const int block[
         if (it != od_idx.end()) bg.nbr_eo[(size_t)i * 8 + 2 * mu + dir] = it->second;
       }
 
-  for (int snake = 0; snake < 2; ++snake) {
-    const int no = snake ? bg.n_o1 : bg.n_ob, ne = snake ? bg.n_e2 : bg.n_b;
-    const std::array<int, 3> odd = {bg.n_ob, bg.n_o1, bg.n_o1}, even = {bg.n_b, bg.n_e1, bg.n_e2};
-    bg.dense[snake][0] = dense_sites(bg.nbr_oe, no, odd, bg.n_b, bg.nbr_read[snake][0]);
-    bg.dense[snake][1] = dense_sites(bg.nbr_eo, ne, even, no, bg.nbr_read[snake][1]);
-    bg.dense[snake][2] = dense_sites(bg.nbr_oe, no, odd, ne, bg.nbr_read[snake][2]);
-    bg.dense[snake][3] = dense_sites(bg.nbr_eo, bg.n_b, even, no, bg.nbr_read[snake][3]);
-  }
-
   bg.gsite.assign((size_t)bg.nblocks * bg.n_comb, 0);
   bg.gmap_b.assign((size_t)bg.nblocks * bg.n_b, 0);
   for (int b = 0; b < bg.nblocks; ++b) {
@@ -206,6 +197,15 @@ void build_block_geometry(BlockGeometry &bg, const int dims[4], const int block[
     for (int i = 0; i < bg.n_o1; ++i) bg.gsite[(size_t)b * bg.n_comb + bg.n_e2 + i] = glob(od[i]);
     for (int i = 0; i < bg.n_b; ++i) bg.gmap_b[(size_t)b * bg.n_b + i] = glob(ev[i]) >> 1;
   }
+}
+
+void find_dense_sites(BlockGeometry &bg, int snake) {
+  const int no = snake ? bg.n_o1 : bg.n_ob, ne = snake ? bg.n_e2 : bg.n_b;
+  const std::array<int, 3> odd = {bg.n_ob, bg.n_o1, bg.n_o1}, even = {bg.n_b, bg.n_e1, bg.n_e2};
+  bg.dense[snake][0] = dense_sites(bg.nbr_oe, no, odd, bg.n_b, bg.nbr_read[snake][0]);
+  bg.dense[snake][1] = dense_sites(bg.nbr_eo, ne, even, no, bg.nbr_read[snake][1]);
+  bg.dense[snake][2] = dense_sites(bg.nbr_oe, no, odd, ne, bg.nbr_read[snake][2]);
+  bg.dense[snake][3] = dense_sites(bg.nbr_eo, bg.n_b, even, no, bg.nbr_read[snake][3]);
 }
 
 }  // namespace dwf

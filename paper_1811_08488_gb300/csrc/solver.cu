@@ -333,7 +333,7 @@ static FieldRef block_ref(const DevBuf &buf, dwf_prec p, int nsite, int Ls, int 
   return f;
 }
 
-BlockPlan *get_block_plan(dwf_ctx *ctx, const int block[4], dwf_prec inner, int nrhs,
+BlockPlan *get_block_plan(dwf_ctx *ctx, const int block[4], dwf_prec inner, int nrhs, int snake,
                           cudaStream_t st) {
   DWF_REQUIRE(inner == DWF_FP32 || inner == DWF_FP16 || inner == DWF_BF16, DWF_ERR_INVALID_ARG,
               "inner precision must be FP32, FP16 or BF16");
@@ -353,9 +353,6 @@ BlockPlan *get_block_plan(dwf_ctx *ctx, const int block[4], dwf_prec inner, int 
     };
     up(bp->nbr_oe, g.nbr_oe);
     up(bp->nbr_eo, g.nbr_eo);
-    for (int sn = 0; sn < 2; ++sn)
-      for (int h = 0; h < 4; ++h)
-        if (!g.nbr_read[sn][h].empty()) up(bp->nbr_read[sn][h], g.nbr_read[sn][h]);
     up(bp->gmap_b, g.gmap_b);
     std::vector<int> own(g.gsite.size());
     const int *L = ctx->act.dims;
@@ -370,6 +367,19 @@ BlockPlan *get_block_plan(dwf_ctx *ctx, const int block[4], dwf_prec inner, int 
   }
   BlockPlan *bp = slot.get();
   const BlockGeometry &g = bp->bg;
+  const int sn = snake ? 1 : 0;
+  if (!bp->have_dense[sn]) {  // the hops' dense sites, for the form of A_s that is used
+    find_dense_sites(bp->bg, sn);
+    for (int h = 0; h < 4; ++h) {
+      std::vector<int> &rd = bp->bg.nbr_read[sn][h];
+      if (rd.empty()) continue;
+      DevBuf &d = bp->nbr_read[sn][h];
+      d.ensure(rd.size() * sizeof(int));
+      DWF_CUDA_TRY(cudaMemcpy(d.p, rd.data(), d.bytes, cudaMemcpyHostToDevice));
+      std::vector<int>().swap(rd);
+    }
+    bp->have_dense[sn] = true;
+  }
   if (!bp->links_valid) {
     const dwf_prec lp = inner == DWF_FP32 ? DWF_FP32 : DWF_FP16;
     bp->link_bstride = (long long)g.n_comb * 4 * (long long)link_record_bytes(lp, ctx->act.recon12);
@@ -852,7 +862,7 @@ dwf_status solve(dwf_ctx *ctx, void *x, const void *b, int nrhs, const double *m
   SolverPlan *sp = get_solver_plan(ctx, lo, nrhs);
   BlockPlan *bp = prm->inner_iters == 0
                       ? nullptr
-                      : get_block_plan(ctx, prm->block, prm->inner, nrhs, st);
+                      : get_block_plan(ctx, prm->block, prm->inner, nrhs, prm->snake, st);
   const int Vh = ctx->geo.Vh, Ls = ctx->act.Ls;
 
   SolveSetup S{ctx, sp, bp, prm, mf, nrhs};

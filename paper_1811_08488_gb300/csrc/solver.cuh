@@ -53,6 +53,7 @@ struct BlockPlan {
   int Ls = 0;
   DevBuf nbr_oe, nbr_eo, gmap_b, gowner;
   DevBuf nbr_read[2][4];  // BlockGeometry::nbr_read
+  bool have_dense[2] = {false, false};
   DevBuf links;
   long long link_bstride = 0;
   DevBuf r, p, Ap, x, u1, y, u2, w2;
@@ -65,7 +66,7 @@ struct BlockPlan {
   bool stop_active = false;  // the inner residual stop is on for the launches being built
 };
 
-BlockPlan *get_block_plan(dwf_ctx *ctx, const int block[4], dwf_prec inner, int nrhs,
+BlockPlan *get_block_plan(dwf_ctx *ctx, const int block[4], dwf_prec inner, int nrhs, int snake,
                           cudaStream_t st);
 // out = (+)_s A_s p on the plan's block vectors (p -> Ap), optional <p, Ap>;
 // schur = 1: the blocks of the symmetric form's normal operator.
