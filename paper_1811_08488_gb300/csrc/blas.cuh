@@ -75,9 +75,11 @@ void solve_post_ru(OuterScalars *scal, SolveCtl *ctl, const int *skip_ru, int *s
 int outer_ctas();
 
 void block_gather(dwf_prec in, const BlockArgs &B, int nrhs, cudaStream_t st);
-void block_xr(dwf_prec in, const BlockArgs &B, int last, int nrhs, cudaStream_t st);
+// first: the first of the inner iterations; the last one's x is in the scatter (only:
+// the one iteration there is)
+void block_xr(dwf_prec in, const BlockArgs &B, int first, int nrhs, cudaStream_t st);
 void block_p(dwf_prec in, const BlockArgs &B, int nrhs, cudaStream_t st);
-void block_scatter(const BlockArgs &B, int nrhs, cudaStream_t st);
+void block_scatter(dwf_prec in, const BlockArgs &B, int only, int nrhs, cudaStream_t st);
 void block_export(dwf_prec in, const BlockArgs &B, const FieldRef &src, int nrhs,
                   cudaStream_t st);
 int block_tiles(int n_b, int Ls);

@@ -602,11 +602,11 @@ void block_precondition(dwf_ctx *ctx, BlockPlan *bp, char *z, const char *r, int
   block_gather(bp->inner, B, nrhs, st);
   for (int it = 0; it < k; ++it) {
     block_apply_A(ctx, bp, snake, nrhs, mf, true, skip, st, schur);
-    const int last = it == k - 1;
-    block_xr(bp->inner, B, last, nrhs, st);
-    if (!last) block_p(bp->inner, B, nrhs, st);
+    if (it == k - 1) break;  // the last update of x is the scatter's
+    block_xr(bp->inner, B, it == 0, nrhs, st);
+    block_p(bp->inner, B, nrhs, st);
   }
-  block_scatter(B, nrhs, st);
+  block_scatter(bp->inner, B, k == 1, nrhs, st);
   bp->stop_active = false;
 }
 

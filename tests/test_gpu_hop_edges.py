@@ -92,3 +92,25 @@ def test_nan_stays_with_the_sites_that_use_it(dagger):
     far = (dist(t, 4, 8) + dist(z, 1, 4) + dist(y, 2, 4) + dist(x, 2 + (4 + 1 + 2) % 2, 8)) > 2
     assert not bad[far].any()
     assert bad.any()
+
+
+@pytest.mark.parametrize("inner", ["fp32", "fp16"])
+@pytest.mark.parametrize("k", [1, 2, 3])
+@pytest.mark.parametrize("inner_tol", [0.0, 1e-6])
+def test_block_solve_starts_from_zero(inner, k, inner_tol):
+    """The blocks are solved apart: with the residual of one block set to zero its
+    solution is zero, whatever an earlier call left in the plan, and the others'
+    is bit for bit what it was."""
+    S = Setup((8, 4, 4, 8), 6, seed=11)
+    src = S.source(96)
+    prm = dwf().default_params(block=(4, 4, 4, 4), inner=inner, inner_iters=k, inner_tol=inner_tol)
+    z = S.ctx.new_field("fp32")
+    S.ctx.block_precond(z, S.to_native([src], "fp32"), prm, [0.05])
+    full = S.from_native(z, "fp32", 1)[0]
+    cut = src.copy()
+    cut[:, 4:, :, :, 2:] = 0  # x >= 4, t >= 4: the last of the four blocks
+    S.ctx.block_precond(z, S.to_native([cut], "fp32"), prm, [0.05])
+    got = S.from_native(z, "fp32", 1)[0]
+    assert (got[:, 4:, :, :, 2:] == 0).all() and (full != 0).any()
+    got[:, 4:, :, :, 2:] = full[:, 4:, :, :, 2:]
+    assert np.array_equal(got, full)
