@@ -891,9 +891,13 @@ static void launch_t(const HopParams &P0, int nrhs, cudaStream_t st, dwf_prec pr
   if (grid.x == 0) return;
   if constexpr (!std::is_same<S, F64>::value) {
     if (hop_pairs(P.Ls, prec)) {
-      // the dense sites (whole CTAs of them), then the others
+      // the dense sites (whole CTAs of them), then the others. The second launch costs
+      // about 2 us in the loop graph and the dense form saves a fifth (FP16 hop 1,
+      // 8^3 x 16 blocks of 16^3 x 32 x 12, 3280 dense CTAs: 132 us in one launch, 77
+      // + 30 in two), so fewer than two waves of dense CTAs go with the others.
       const int n_out = P.n_out;
-      const int nd = std::min(n_out, (P.n_dense + nsites - 1) / nsites * nsites);
+      int nd = std::min(n_out, (P.n_dense + nsites - 1) / nsites * nsites);
+      if (nd < n_out && (long long)(nd / nsites) * P.nblocks * nrhs < 2 * 152 * 4) nd = 0;
       if (nd > 0) {
         P.n_out = nd;
         grid.x = (nd + nsites - 1) / nsites;
