@@ -44,33 +44,42 @@ __device__ __forceinline__ uint4 pack8(const float *v, float scl) {
   return q;
 }
 
+// A word of shared memory, or of a field that the kernel also writes (PLAIN), or of
+// global memory that stays as it is for the whole kernel (read-only load).
+template <bool PLAIN, class T>
+__device__ __forceinline__ T ldp(const T *p) {
+  if constexpr (PLAIN) return *p;
+  else return __ldg(p);
+}
+
 // Native layout of one right-hand side (of one block): element e = site*Ls + s,
 // 16-byte chunk c of element e at chunk index c * cs + e with cs = nsite*Ls
 // (chunk-major), so the chunk c of consecutive (site, s) is contiguous and a
 // warp's load of one chunk is a contiguous 512-byte segment. FP16/BF16 scales
-// are one float per element at byte offset soff.
-template <class S>
+// are one float per element at byte offset soff. PLAIN: the kernel may write the
+// field that it reads.
+template <class S, bool PLAIN = false>
 __device__ __forceinline__ void load24(const char *base, long long soff, int cs, int e,
                                        typename S::R *v) {
   if constexpr (std::is_same<S, F32>::value) {
     const float4 *p = reinterpret_cast<const float4 *>(base) + e;
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      float4 q = __ldg(p + (size_t)k * cs);
+      float4 q = ldp<PLAIN>(p + (size_t)k * cs);
       v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
     }
   } else if constexpr (std::is_same<S, F64>::value) {
     const double2 *p = reinterpret_cast<const double2 *>(base) + e;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      double2 q = __ldg(p + (size_t)k * cs);
+      double2 q = ldp<PLAIN>(p + (size_t)k * cs);
       v[2 * k] = q.x; v[2 * k + 1] = q.y;
     }
   } else {
     const uint4 *p = reinterpret_cast<const uint4 *>(base) + e;
-    const float scl = __ldg(reinterpret_cast<const float *>(base + soff) + e);
+    const float scl = ldp<PLAIN>(reinterpret_cast<const float *>(base + soff) + e);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) unpack8<S>(__ldg(p + (size_t)k * cs), v + 8 * k);
+    for (int k = 0; k < 3; ++k) unpack8<S>(ldp<PLAIN>(p + (size_t)k * cs), v + 8 * k);
 #pragma unroll
     for (int k = 0; k < 24; ++k) v[k] *= scl;
   }
@@ -142,11 +151,19 @@ __device__ __forceinline__ void store24(char *base, long long soff, int cs, int 
 // word, moved with a single 256-bit load or store (sm_100 and later). A warp
 // request of 32 such words is one contiguous kilobyte.
 // ---------------------------------------------------------------------------
+template <bool PLAIN = false>
 __device__ __forceinline__ void ldg256(const void *p, uint32_t (&a)[8]) {
-  asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]),
-                 "=r"(a[6]), "=r"(a[7])
-               : "l"(p));
+  if constexpr (PLAIN)
+    asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]),
+                   "=r"(a[6]), "=r"(a[7])
+                 : "l"(p)
+                 : "memory");
+  else
+    asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]),
+                   "=r"(a[6]), "=r"(a[7])
+                 : "l"(p));
 }
 __device__ __forceinline__ void stg256(void *p, const uint32_t (&a)[8]) {
   asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(a[0]),
@@ -155,7 +172,8 @@ __device__ __forceinline__ void stg256(void *p, const uint32_t (&a)[8]) {
 }
 
 // Load the 24 reals of elements e (v0) and e+1 (v1); e even. FP32/FP16/BF16.
-template <class S>
+// PLAIN as in load24.
+template <class S, bool PLAIN = false>
 __device__ __forceinline__ void load24x2(const char *base, long long soff, int cs, int e,
                                          float *v0, float *v1) {
   const uint4 *p = reinterpret_cast<const uint4 *>(base) + e;
@@ -163,7 +181,7 @@ __device__ __forceinline__ void load24x2(const char *base, long long soff, int c
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
       uint32_t a[8];
-      ldg256(p + (size_t)k * cs, a);
+      ldg256<PLAIN>(p + (size_t)k * cs, a);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         v0[4 * k + i] = __uint_as_float(a[i]);
@@ -171,11 +189,11 @@ __device__ __forceinline__ void load24x2(const char *base, long long soff, int c
       }
     }
   } else {
-    const float2 scl = __ldg(reinterpret_cast<const float2 *>(base + soff) + e / 2);
+    const float2 scl = ldp<PLAIN>(reinterpret_cast<const float2 *>(base + soff) + e / 2);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       uint32_t a[8];
-      ldg256(p + (size_t)k * cs, a);
+      ldg256<PLAIN>(p + (size_t)k * cs, a);
       unpack8<S>(make_uint4(a[0], a[1], a[2], a[3]), v0 + 8 * k);
       unpack8<S>(make_uint4(a[4], a[5], a[6], a[7]), v1 + 8 * k);
     }
@@ -295,13 +313,6 @@ __device__ __forceinline__ void reconstruct_row2(R *u, R sg) {
   }
 }
 
-// One word (or its start) of a link record in global or shared memory.
-template <bool SMEM, class T>
-__device__ __forceinline__ T ldl(const T *p) {
-  if constexpr (SMEM) return *p;
-  else return __ldg(p);
-}
-
 // Load the link record whose word 0 is at w; word k is at w[k * ws] (the
 // chunk-major link layout: ws = number of link owners). recon: the record
 // holds two rows and a sign (reconstruct-12, FP32/FP16/BF16 only). SMEM: the
@@ -312,38 +323,38 @@ __device__ __forceinline__ void load_link(const uint4 *w, size_t ws, typename S:
   if constexpr (std::is_same<S, F64>::value) {
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-      const double2 q = ldl<SMEM>(reinterpret_cast<const double2 *>(w + k * ws));
+      const double2 q = ldp<SMEM>(reinterpret_cast<const double2 *>(w + k * ws));
       u[2 * k] = q.x; u[2 * k + 1] = q.y;
     }
   } else if constexpr (std::is_same<S, F32>::value) {
     if (recon) {
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        const float4 q = ldl<SMEM>(reinterpret_cast<const float4 *>(w + k * ws));
+        const float4 q = ldp<SMEM>(reinterpret_cast<const float4 *>(w + k * ws));
         u[4 * k] = q.x; u[4 * k + 1] = q.y; u[4 * k + 2] = q.z; u[4 * k + 3] = q.w;
       }
-      reconstruct_row2<float>(u, ldl<SMEM>(reinterpret_cast<const float *>(w + 3 * ws)));
+      reconstruct_row2<float>(u, ldp<SMEM>(reinterpret_cast<const float *>(w + 3 * ws)));
     } else {
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const float4 q = ldl<SMEM>(reinterpret_cast<const float4 *>(w + k * ws));
+        const float4 q = ldp<SMEM>(reinterpret_cast<const float4 *>(w + k * ws));
         u[4 * k] = q.x; u[4 * k + 1] = q.y; u[4 * k + 2] = q.z; u[4 * k + 3] = q.w;
       }
-      const float2 q = ldl<SMEM>(reinterpret_cast<const float2 *>(w + 4 * ws));
+      const float2 q = ldp<SMEM>(reinterpret_cast<const float2 *>(w + 4 * ws));
       u[16] = q.x; u[17] = q.y;
     }
   } else {
     if (recon) {
       float t[16];
-      unpack8<F16>(ldl<SMEM>(w), t);
-      unpack8<F16>(ldl<SMEM>(w + ws), t + 8);
+      unpack8<F16>(ldp<SMEM>(w), t);
+      unpack8<F16>(ldp<SMEM>(w + ws), t + 8);
 #pragma unroll
       for (int k = 0; k < 12; ++k) u[k] = t[k];
       reconstruct_row2<float>(u, t[12]);
     } else {
       float t[24];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) unpack8<F16>(ldl<SMEM>(w + k * ws), t + 8 * k);
+      for (int k = 0; k < 3; ++k) unpack8<F16>(ldp<SMEM>(w + k * ws), t + 8 * k);
 #pragma unroll
       for (int k = 0; k < 18; ++k) u[k] = t[k];
     }

@@ -14,8 +14,8 @@ namespace dwf {
 // Grid z runs over nrhs * coef_div fields of nsite sites (block-local fields
 // of every block are laid out like right-hand sides); field z uses the
 // coefficients of right-hand side z / coef_div (skipped when its skip flag is
-// set). A CTA reads its sites before it
-// writes them, so out may equal in.
+// set). A CTA reads its sites before it writes them and no other CTA's, and by plain
+// loads, so out may equal in.
 template <class S, bool DAG>
 __global__ void __launch_bounds__(256) ls_kernel(char *out, const char *in, long long rstride,
                                                  long long soff, int nsite, int Ls, int inv,
@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(256) ls_kernel(char *out, const char *in, long
   char *op = out + rhs * rstride;
   if (active) {
     R v[24];
-    load24<S>(ip, soff, nsite * Ls, site * Ls + s, v);
+    load24<S, true>(ip, soff, nsite * Ls, site * Ls + s, v);
 #pragma unroll
     for (int k = 0; k < 24; ++k) T[(sl * 24 + k) * col + s] = v[k];
   }
@@ -58,8 +58,8 @@ __global__ void __launch_bounds__(256) ls_kernel(char *out, const char *in, long
 // slices of a site in 256-bit loads and the operator runs on the lanes of the site
 // (ls_lanes), so nothing waits at a barrier and every load of a warp is a contiguous
 // kilobyte. HBM-bound: M_5^-1 of 16 right-hand sides on 16^3 x 32 x 12, 2.42 GB, 344 us
-// (7.0 TB/s) against 516 us with ls_kernel. It writes only what its own warp has
-// read: out may equal in.
+// (7.0 TB/s) against 516 us with ls_kernel. A warp reads its own sites only, by plain
+// loads, before it writes them (lanes without a site load nothing): out may equal in.
 template <bool DAG>
 __global__ void __launch_bounds__(128) ls2_kernel(char *out, const char *in, long long rstride,
                                                   int nsite, int Ls, int inv, int coef_div,
@@ -71,9 +71,14 @@ __global__ void __launch_bounds__(128) ls2_kernel(char *out, const char *in, lon
   const int jp = lane % np, slw = lane / np;
   const int site = (blockIdx.x * 4 + (threadIdx.x >> 5)) * spw + slw;
   const bool active = slw < spw && site < nsite;
-  const int e = (active ? site : 0) * Ls + 2 * jp;
+  const int e = site * Ls + 2 * jp;
   float a0[24], a1[24];
-  load24x2<F32>(in + rhs * rstride, 0, nsite * Ls, e, a0, a1);
+  if (active) {
+    load24x2<F32, true>(in + rhs * rstride, 0, nsite * Ls, e, a0, a1);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 24; ++k) a0[k] = a1[k] = 0.f;
+  }
   ls_lanes<DAG>(a0, a1, inv != 0, Ls, np, jp, lane, cf.f, pair_lanes(lane, jp, np, cf.f.mf));
   if (active) store24x2<F32>(out + rhs * rstride, 0, nsite * Ls, e, a0, a1);
 }
