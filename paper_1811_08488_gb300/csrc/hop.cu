@@ -574,6 +574,12 @@ __device__ __forceinline__ void load_dir2(DirIn &in2, const char *in, long long 
     load24x2<S>(in, soff, cs, e, in2.v0, in2.v1);
 }
 
+__device__ __forceinline__ void zero_dir2(DirIn &d) {
+#pragma unroll
+  for (int k = 0; k < 24; ++k) d.v0[k] = d.v1[k] = 0.f;
+  d.sc = make_float2(0.f, 0.f);
+}
+
 // The projected spins of one direction from its loaded input.
 template <class S, int MU, bool FWD, bool DAG, bool PRE>
 __device__ __forceinline__ void dir_project(HalfSpinor &h, const DirIn &d, const LsCoef &cf,
@@ -582,26 +588,31 @@ __device__ __forceinline__ void dir_project(HalfSpinor &h, const DirIn &d, const
   if constexpr (PRE) {
     // M_phi on both slices as packed FMAs: (chi(s0), chi(s0+1)) =
     // b (v(s0), v(s0+1)) + c (shifted neighbours); the outer halves come
-    // from the neighbouring lanes of the same site (all lanes take part). The
-    // wrap factors and the slices' scales are folded into the coefficients.
+    // from the neighbouring lanes of the same site (all lanes take part). FP16/BF16: the
+    // wrap factors and the slices' scales are folded into the coefficients. FP32: the
+    // wrap factor is applied to the outer half; folded in, the coefficients are pairs of
+    // their own in every lane, and M^4 without staged links took 1 to 2 % longer.
     const float b = cf.f.pre_b, c = cf.f.pre_c;
-    float2 bs = bc(b), cu = make_float2(c * pl.fm, c), cl = make_float2(c, c * pl.fp);
+    float2 bs = bc(b), cu = bc(c), cl = bc(c);
     if constexpr (S::kHalf) {
       const float sm = __shfl_sync(0xffffffffu, d.sc.y, pl.up);
       const float sp = __shfl_sync(0xffffffffu, d.sc.x, pl.dn);
       bs = make_float2(b * d.sc.x, b * d.sc.y);
-      cu = make_float2(cu.x * sm, c * d.sc.x);
-      cl = make_float2(c * d.sc.y, cl.y * sp);
+      cu = make_float2(c * pl.fm * sm, c * d.sc.x);
+      cl = make_float2(c * d.sc.y, c * pl.fp * sp);
     }
+    const float fm = S::kHalf ? 1.f : pl.fm, fp = S::kHalf ? 1.f : pl.fp;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {  // upper: chi(s0) <- s0-1, chi(s0+1) <- s0
       const float w = __shfl_sync(0xffffffffu, d.v1[k], pl.up);
-      v[k] = __ffma2_rn(cu, make_float2(w, d.v0[k]), __fmul2_rn(bs, make_float2(d.v0[k], d.v1[k])));
+      v[k] = __ffma2_rn(cu, make_float2(fm * w, d.v0[k]),
+                        __fmul2_rn(bs, make_float2(d.v0[k], d.v1[k])));
     }
 #pragma unroll
     for (int k = 12; k < 24; ++k) {  // lower: chi(s0) <- s0+1, chi(s0+1) <- s0+2
       const float w = __shfl_sync(0xffffffffu, d.v0[k], pl.dn);
-      v[k] = __ffma2_rn(cl, make_float2(d.v1[k], w), __fmul2_rn(bs, make_float2(d.v0[k], d.v1[k])));
+      v[k] = __ffma2_rn(cl, make_float2(d.v1[k], fp * w),
+                        __fmul2_rn(bs, make_float2(d.v0[k], d.v1[k])));
     }
   } else {
 #pragma unroll
@@ -766,7 +777,8 @@ __device__ __forceinline__ void hop2_body(const HopParams &P) {
   } else {
     // With M_phi on load every lane of the warp takes part in a direction (its
     // halves are exchanged between lanes) and one that no lane has is skipped by
-    // all; otherwise each lane branches on its own neighbour.
+    // all; otherwise each lane branches on its own neighbour. A lane without the
+    // neighbour loads nothing.
     constexpr int LC = link_words<S, RC>();
     const size_t ls = (size_t)P.link_cs;
     const int4 *nb = reinterpret_cast<const int4 *>(P.nbr + (size_t)(active ? site : 0) * 8);
@@ -777,7 +789,10 @@ __device__ __forceinline__ void hop2_body(const HopParams &P) {
     const int j = active ? js[D] : -1;                                                         \
     const bool valid = (unsigned)j < (unsigned)P.in_limit;                                     \
     if (PRE ? __any_sync(0xffffffffu, valid) != 0 : valid) {                                   \
-      HOP_LOAD(valid ? j : 0);                                                                 \
+      if (!PRE || valid)                                                                       \
+        HOP_LOAD(j);                                                                           \
+      else                                                                                     \
+        zero_dir2(d);                                                                          \
       HOP_PROJECT(D)                                                                           \
       if (valid)                                                                               \
         dir_add<S, (D) / 2, ((D) & 1) == 0, DAG, PRE, RC, false>(                              \
