@@ -155,8 +155,9 @@ struct HopParams {
   const int *nbr = nullptr;  // [n_out][8], direction 2*mu + (0 fwd, 1 bwd)
   int n_out = 0;             // output sites per block
   int in_limit = 0;          // inputs with index >= in_limit are zero
-  int n_dense = 0;           // sites below it run all eight directions (see dense_sites),
-  const int *nbr_read = nullptr;  // reading these neighbours (nbr with the absent ones replaced)
+  int n_dense = 0;           // sites below it may run with staged links (hop_staged_sites),
+  const int *nbr_read = nullptr;  // all eight directions, reading these neighbours: nbr with
+                                  // the absent ones replaced, for all of n_out
   int site_off = 0;          // first output site of the launch (set by the launcher)
   int dirs = 0xff;           // all eight directions (the dense FP32 hop branches on it)
   int xown_limit = 0;        // xown is zero for sites >= xown_limit
@@ -204,17 +205,24 @@ struct BlockGeometry {
   std::vector<int> nbr_oe;  // [n_o1][8]: odd out <- even in (local even index or -1)
   std::vector<int> nbr_eo;  // [n_e2][8]: even out <- odd in (local odd index or -1)
   std::vector<int> gsite;   // [nblocks][n_comb] global lexicographic site of each owner
-  // leading sites of each block hop with all or most neighbours [snake][hop 1..4], and
-  // their neighbours with the absent ones replaced (empty where none is absent)
-  // (filled by find_dense_sites)
+  // [snake][hop 1..4], filled by find_dense_sites: leading sites with all or most
+  // neighbours, and whether no output site of the hop lacks one
   int dense[2][4];
-  std::vector<int> nbr_read[2][4];
+  bool complete[2][4];
   std::vector<int> gmap_b;  // [nblocks][n_b] global even half index of block sites
 };
 
 void build_geometry(Geometry &g, const int dims[4]);
 void build_block_geometry(BlockGeometry &bg, const int dims[4], const int block[4]);
 void find_dense_sites(BlockGeometry &bg, int snake);
+// Output sites, input sites and neighbour table of block hop h + 1.
+struct BlockHop {
+  int n_out, in_limit;
+  const std::vector<int> &nbr;
+};
+BlockHop block_hop(const BlockGeometry &bg, int snake, int h);
+// The neighbours of a block hop with the absent ones replaced by another of the site's.
+std::vector<int> present_neighbours(const BlockHop &hop);
 
 // ---------------------------------------------------------------------------
 // Device buffers
@@ -311,6 +319,9 @@ namespace dwf {
 template <class S>
 void launch_hop(const HopParams &P, int dagger, int pre_mphi, int nrhs, cudaStream_t st);
 int hop_sites_per_cta(int Ls, dwf_prec p);
+int hop_staged_sites(int Ls, dwf_prec p, int dagger, int pre, int n_dense, int n_out,
+                     long long fields, int sms);
+int sm_count();  // SMs of the current device
 size_t hop_smem_bytes(int Ls, dwf_prec p, int epi, int has_x, int recon);
 
 // ls.cu: Ls-local operators (M_5, M_5^-1) on native fields

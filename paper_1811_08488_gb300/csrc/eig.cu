@@ -72,18 +72,6 @@ static int wave_ctas() {
   return n;
 }
 
-// SMs of the current device.
-static int sm_count() {
-  constexpr int kDevices = 64;
-  static std::atomic<int> cache[kDevices];  // 0 until read
-  int dev = 0, n = 0;
-  DWF_CUDA_TRY(cudaGetDevice(&dev));
-  if (dev < kDevices && (n = cache[dev].load(std::memory_order_relaxed)) > 0) return n;
-  DWF_CUDA_TRY(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
-  if (dev < kDevices) cache[dev].store(n, std::memory_order_relaxed);
-  return n;
-}
-
 // CTAs per tile: one wave over all tiles (at least one CTA per tile), at most
 // one CTA per `per_cta` work items of a tile, and at most kEigCtas in all
 // (the partial-sum scratch holds kEigCtas CTAs).

@@ -59,41 +59,50 @@ static inline int side1(int u, int bl, int L) {
   return (u - bl + 1 <= L - u) ? 1 : 2;
 }
 
-// How many of the leading n_out sites run all eight directions of a block hop: ring
-// after ring (the sites at distance 0, 1, 2 end at `ends`) as long as a ring's sites
-// have 5 of 8 neighbours or more on average. A direction that is left out saves its
-// arithmetic, one that always runs is loaded ahead of it. In 12^3 x 16 blocks the
-// even sites at distance 0, 1 and 2 have 8, 7 and 1 to 2 odd neighbours in the
-// region (FP16 hop 2: 427 us with all sites run by tests, 418 with distance 0 run
-// densely). In 2^4 blocks every site has 4 of its own block.
-// read: the neighbours with the absent ones replaced by another of the site's
-// (left empty when none is absent).
-static int dense_sites(const std::vector<int> &nbr, int n_out, std::array<int, 3> ends,
-                       int in_limit, std::vector<int> &read) {
-  auto has = [&](size_t i) { return nbr[i] >= 0 && nbr[i] < in_limit; };
-  auto count = [&](int from, int to) {
-    long long have = 0;
-    for (size_t i = (size_t)from * 8; i < (size_t)to * 8; ++i) have += has(i);
-    return have;
-  };
-  int n = 0;
-  for (int e : ends) {
-    e = std::min(e, n_out);
-    if (e <= n) continue;
-    if (count(n, e) < 5LL * (e - n)) break;
-    n = e;
+BlockHop block_hop(const BlockGeometry &bg, int snake, int h) {
+  const int no = snake ? bg.n_o1 : bg.n_ob, ne = snake ? bg.n_e2 : bg.n_b;
+  if (h % 2 == 0) return {no, h == 0 ? bg.n_b : ne, bg.nbr_oe};
+  return {h == 1 ? ne : bg.n_b, no, bg.nbr_eo};
+}
+
+// Leading output sites of a block hop that may run all eight directions with staged
+// links: ring after ring (the sites at distance 0, 1, 2) as long as a ring's sites have 5
+// of 8 neighbours or more on average. A direction that is left out saves its
+// arithmetic, one that always runs is loaded ahead of it. In 12^3 x 16 blocks the even
+// sites at distance 0, 1 and 2 have 8, 7 and 1 to 2 odd neighbours in the region. In 2^4
+// blocks every site has 4 of its own block.
+void find_dense_sites(BlockGeometry &bg, int snake) {
+  for (int h = 0; h < 4; ++h) {
+    const BlockHop hop = block_hop(bg, snake, h);
+    const std::array<int, 3> ends = h % 2 == 0 ? std::array<int, 3>{bg.n_ob, bg.n_o1, bg.n_o1}
+                                               : std::array<int, 3>{bg.n_b, bg.n_e1, bg.n_e2};
+    int from = 0, dense = 0;
+    bool all = true, growing = true;
+    for (int e : ends) {
+      e = std::min(e, hop.n_out);
+      long long have = 0;
+      for (size_t i = (size_t)from * 8; i < (size_t)e * 8; ++i)
+        have += (unsigned)hop.nbr[i] < (unsigned)hop.in_limit;
+      all = all && have == 8LL * (e - from);
+      growing = growing && have >= 5LL * (e - from);
+      if (growing) dense = e;
+      from = e;
+    }
+    bg.dense[snake][h] = dense;
+    bg.complete[snake][h] = all;
   }
-  // whole CTAs of sites are run, so the table covers all
-  if (n == 0 || count(0, n_out) == 8LL * n_out) return n;
-  read.assign(nbr.begin(), nbr.begin() + (size_t)n_out * 8);
-  for (size_t s = 0; s < (size_t)n_out; ++s) {
+}
+
+std::vector<int> present_neighbours(const BlockHop &hop) {
+  std::vector<int> read(hop.nbr.begin(), hop.nbr.begin() + (size_t)hop.n_out * 8);
+  for (size_t s = 0; s < read.size(); s += 8) {
     int some = 0;
     for (int k = 0; k < 8; ++k)
-      if (has(8 * s + k)) some = nbr[8 * s + k];
+      if ((unsigned)read[s + k] < (unsigned)hop.in_limit) some = read[s + k];
     for (int k = 0; k < 8; ++k)
-      if (!has(8 * s + k)) read[8 * s + k] = some;
+      if ((unsigned)read[s + k] >= (unsigned)hop.in_limit) read[s + k] = some;
   }
-  return n;
+  return read;
 }
 
 void build_block_geometry(BlockGeometry &bg, const int dims[4], const int block[4]) {
@@ -197,15 +206,6 @@ void build_block_geometry(BlockGeometry &bg, const int dims[4], const int block[
     for (int i = 0; i < bg.n_o1; ++i) bg.gsite[(size_t)b * bg.n_comb + bg.n_e2 + i] = glob(od[i]);
     for (int i = 0; i < bg.n_b; ++i) bg.gmap_b[(size_t)b * bg.n_b + i] = glob(ev[i]) >> 1;
   }
-}
-
-void find_dense_sites(BlockGeometry &bg, int snake) {
-  const int no = snake ? bg.n_o1 : bg.n_ob, ne = snake ? bg.n_e2 : bg.n_b;
-  const std::array<int, 3> odd = {bg.n_ob, bg.n_o1, bg.n_o1}, even = {bg.n_b, bg.n_e1, bg.n_e2};
-  bg.dense[snake][0] = dense_sites(bg.nbr_oe, no, odd, bg.n_b, bg.nbr_read[snake][0]);
-  bg.dense[snake][1] = dense_sites(bg.nbr_eo, ne, even, no, bg.nbr_read[snake][1]);
-  bg.dense[snake][2] = dense_sites(bg.nbr_oe, no, odd, ne, bg.nbr_read[snake][2]);
-  bg.dense[snake][3] = dense_sites(bg.nbr_eo, bg.n_b, even, no, bg.nbr_read[snake][3]);
 }
 
 }  // namespace dwf

@@ -29,9 +29,10 @@
 // instructions per site instead of 553, 660 us for the adjoint); an L2 prefetch
 // of the rows that come next (535 us).
 //
-// A launch runs `dense` sites, which have all or most neighbours, in this form.
-// A block's outer ring, with one or two neighbours each, runs direction by
-// direction with the links read where they are (DENSE = false).
+// The other form of the kernel (DENSE = false) runs direction by direction, leaves out
+// those that no lane has, and reads the links where they are: for the outer ring of a
+// block's region, whose sites have one or two neighbours, and where staging does not
+// pay (hop_staged_sites has the rule and its measurements).
 //
 // hop_kernel (FP64 fields, odd Ls): one thread per output (site, s), the Ls
 // epilogue walks columns in shared memory.
@@ -45,6 +46,7 @@
 // chi_u(s) = b psi_u(s) + c psi_u(s-1), chi_l(s) = b psi_l(s) + c psi_l(s+1),
 // with the wrap factor -m_f.
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "device_common.cuh"
@@ -374,6 +376,8 @@ __global__ void __launch_bounds__(256) hop_kernel(const __grid_constant__ HopPar
   hop_body<S, DAG, PRE, RC>(P);
   prof_exit(P);
 }
+
+constexpr int kHopCtas = 4;  // CTAs of hop2_kernel per SM (128 registers a thread)
 
 // ---------------------------------------------------------------------------
 // Two slices per thread: thread (site, s0 = 2j) computes s0 and s0 + 1. Chunk c
@@ -854,10 +858,21 @@ __device__ __forceinline__ void hop2_body(const HopParams &P) {
 }
 
 template <class S, bool DAG, bool PRE, bool RC, bool EPI, bool DENSE>
-__global__ void __launch_bounds__(128, 4) hop2_kernel(const __grid_constant__ HopParams P) {
+__global__ void __launch_bounds__(128, kHopCtas) hop2_kernel(const __grid_constant__ HopParams P) {
   prof_enter(P);
   hop2_body<S, DAG, PRE, RC, EPI, DENSE>(P);
   prof_exit(P);
+}
+
+int sm_count() {
+  constexpr int kDevices = 64;
+  static std::atomic<int> cache[kDevices];  // 0 until read
+  int dev = 0, n = 0;
+  DWF_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < kDevices && (n = cache[dev].load(std::memory_order_relaxed)) > 0) return n;
+  DWF_CUDA_TRY(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+  if (dev < kDevices) cache[dev].store(n, std::memory_order_relaxed);
+  return n;
 }
 
 // Two slices per thread for FP32/FP16/BF16 with even Ls; one otherwise.
@@ -875,6 +890,48 @@ int hop_sites_per_cta(int Ls, dwf_prec p) {
   for (int n = most; n >= 1 && 2 * n >= most; --n)
     if (n * lanes(best) > best * lanes(n)) best = n;
   return best;
+}
+
+// How many leading output sites of a hop (0, n_out, or whole CTAs of the n_dense that
+// have all or most neighbours) run with staged links, the others direction by direction;
+// fields: blocks x right-hand sides. Measured with against without staged links, 1 wave =
+// 4 CTAs on every SM:
+// - A staged link serves the Ls/2 lanes of a site. With one lane the copy takes 82 KB of
+//   the SM's shared memory and two CTAs fit, with two lanes it saves little (24^3 x 48, FP16
+//   adjoint: 112 against 53 us with Ls = 2, 100 against 91 with Ls = 4).
+// - All sites, FP16/BF16: with M_phi on load it pays from two lanes on at every size (24^3 x
+//   48: 117 against 127 us with Ls = 4, 364 against 467 with Ls = 16), the hops without it
+//   from four lanes on (Ls = 8: 158 against 168, Ls = 6: 140 against 138).
+// - All sites, FP32: below two waves the wait for the links before the first direction
+//   shows (16^4, Ls = 6, 1.35 waves: 22.8 against 20.7 us, adjoint 19.3 against 16.7;
+//   16^3 x 32, 2.7 waves: 43.2 against 47.0 and 37.3 against 38.3), but not from six lanes
+//   on, with M_phi on load twelve (12^3 x 16, Ls = 24: 34.2 against 37.1, adjoint 26.9
+//   against 28.9).
+// - Some sites, then a second launch (about 2 us, and a last wave of its own) for the rest;
+//   k = 3 preconditioner, FP16 hop 1 (M_phi on load): two launches gain 1 % from 3 waves
+//   (8^3 x 16 blocks of 16^3 x 32, Ls = 8: 3.4 waves), lose 1 to 3 % below (2.7 and 1.4).
+//   FP32 hop 2: gains 1 to 2 % from 24 waves (12^3 x 16 blocks, Ls = 10), loses 1 to 2 % at 6
+//   to 10. FP16 hop 2 and FP32 hop 1: no gain at any size.
+int hop_staged_sites(int Ls, dwf_prec p, int dagger, int pre, int n_dense, int n_out,
+                     long long fields, int sms) {
+  if (!hop_pairs(Ls, p) || n_dense <= 0) return 0;
+  const int lanes = Ls / 2, nsites = hop_sites_per_cta(Ls, p);
+  const int ctas = (std::min(n_dense, n_out) + nsites - 1) / nsites;
+  const int nd = std::min(n_out, ctas * nsites);
+  const bool half = p != DWF_FP32;
+  int fewest, waves;  // lanes of a site and waves of CTAs that it takes
+  if (nd < n_out) {
+    if (dagger || half != (pre != 0)) return 0;
+    fewest = 3;
+    waves = half ? 3 : 24;
+  } else if (half) {
+    fewest = pre ? 2 : 4;
+    waves = 0;
+  } else {
+    fewest = 3;
+    waves = lanes >= (pre ? 12 : 6) ? 0 : 2;
+  }
+  return lanes >= fewest && ctas * fields >= (long long)waves * kHopCtas * sms ? nd : 0;
 }
 
 size_t hop_smem_bytes(int Ls, dwf_prec p, int epi, int has_x, int recon) {
@@ -911,13 +968,10 @@ static void launch_t(const HopParams &P0, int nrhs, cudaStream_t st, dwf_prec pr
   if (grid.x == 0) return;
   if constexpr (!std::is_same<S, F64>::value) {
     if (hop_pairs(P.Ls, prec)) {
-      // the dense sites (whole CTAs of them), then the others. The second launch costs
-      // about 2 us in the loop graph and the dense form saves a fifth (FP16 hop 1,
-      // 8^3 x 16 blocks of 16^3 x 32 x 12, 3280 dense CTAs: 132 us in one launch, 77
-      // + 30 in two), so fewer than two waves of dense CTAs go with the others.
+      // the sites with staged links (whole CTAs of them), then the others
       const int n_out = P.n_out;
-      int nd = std::min(n_out, (P.n_dense + nsites - 1) / nsites * nsites);
-      if (nd < n_out && (long long)(nd / nsites) * P.nblocks * nrhs < 2 * 152 * 4) nd = 0;
+      const int nd = hop_staged_sites(P.Ls, prec, DAG, PRE, P.n_dense, n_out,
+                                      (long long)P.nblocks * nrhs, sm_count());
       if (nd > 0) {
         P.n_out = nd;
         grid.x = (nd + nsites - 1) / nsites;
@@ -970,20 +1024,13 @@ void launch_hop(const HopParams &P, int dagger, int pre_mphi, int nrhs, cudaStre
     launch_t<S, false, false, false>(P, nrhs, st, p);
 }
 
-// Allow the hop kernels more than 48 KB of dynamic shared memory. Called once per device before any launch
-// (and so before any stream capture).
+// Allow the one-slice hop kernels more than 48 KB of dynamic shared memory (staged links
+// take 41 KB at most). Called once per device before any launch (and so before any
+// stream capture).
 template <class K>
 static void allow_big_smem(K *kernel) {
   DWF_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     200 * 1024));
-}
-template <class S, bool RC>
-static void prepare_two() {
-  allow_big_smem(hop2_kernel<S, false, false, RC, false, true>);
-  allow_big_smem(hop2_kernel<S, false, false, RC, true, true>);
-  allow_big_smem(hop2_kernel<S, false, true, RC, false, true>);
-  allow_big_smem(hop2_kernel<S, false, true, RC, true, true>);
-  allow_big_smem(hop2_kernel<S, true, false, RC, true, true>);
 }
 template <class S>
 static void prepare_one() {
@@ -994,8 +1041,6 @@ static void prepare_one() {
     allow_big_smem(hop_kernel<S, false, false, true>);
     allow_big_smem(hop_kernel<S, false, true, true>);
     allow_big_smem(hop_kernel<S, true, false, true>);
-    prepare_two<S, false>();
-    prepare_two<S, true>();
   }
 }
 void prepare_kernels() {

@@ -6,6 +6,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <sstream>
+#include <utility>
 
 #include "solver.cuh"
 
@@ -368,17 +369,25 @@ BlockPlan *get_block_plan(dwf_ctx *ctx, const int block[4], dwf_prec inner, int 
   BlockPlan *bp = slot.get();
   const BlockGeometry &g = bp->bg;
   const int sn = snake ? 1 : 0;
-  if (!bp->have_dense[sn]) {  // the hops' dense sites, for the form of A_s that is used
+  if (!bp->have_dense[sn]) {
     find_dense_sites(bp->bg, sn);
-    for (int h = 0; h < 4; ++h) {
-      std::vector<int> &rd = bp->bg.nbr_read[sn][h];
-      if (rd.empty()) continue;
-      DevBuf &d = bp->nbr_read[sn][h];
-      d.ensure(rd.size() * sizeof(int));
-      DWF_CUDA_TRY(cudaMemcpy(d.p, rd.data(), d.bytes, cudaMemcpyHostToDevice));
-      std::vector<int>().swap(rd);
-    }
     bp->have_dense[sn] = true;
+  }
+  // the neighbours that a hop reads, where one is absent and the hop runs with staged
+  // links for this form of A_s and number of right-hand sides (hop 1 has M_phi on load,
+  // 3 and 4 are adjoint)
+  for (int h = 0; h < 4; ++h) {
+    const BlockHop hop = block_hop(g, sn, h);
+    if (g.complete[sn][h] || bp->nbr_read[sn][h].p ||
+        hop_staged_sites(Ls, inner, h >= 2, h == 0, g.dense[sn][h], hop.n_out,
+                         (long long)g.nblocks * nrhs, sm_count()) == 0)
+      continue;
+    const std::vector<int> rd = present_neighbours(hop);
+    DevBuf buf;
+    buf.ensure(rd.size() * sizeof(int));
+    DWF_CUDA_TRY(cudaMemcpy(buf.p, rd.data(), buf.bytes, cudaMemcpyHostToDevice));
+    std::swap(bp->nbr_read[sn][h].p, buf.p);  // (kept only once it is filled)
+    std::swap(bp->nbr_read[sn][h].bytes, buf.bytes);
   }
   if (!bp->links_valid) {
     const dwf_prec lp = inner == DWF_FP32 ? DWF_FP32 : DWF_FP16;
@@ -447,8 +456,9 @@ void block_apply_A(dwf_ctx *ctx, BlockPlan *bp, int snake, int nrhs, const doubl
   const int odd_in = snake ? g.n_o1 : g.n_ob;
   // the neighbour table of block hop h + 1 and its dense sites
   auto sites = [&](HopParams &P, int h, const DevBuf &nbr) {
-    const DevBuf &rd = bp->nbr_read[snake ? 1 : 0][h];
-    P.n_dense = g.dense[snake ? 1 : 0][h];
+    const int sn = snake ? 1 : 0;
+    const DevBuf &rd = bp->nbr_read[sn][h];
+    P.n_dense = rd.p || g.complete[sn][h] ? g.dense[sn][h] : 0;
     P.nbr = nbr.as<int>();
     P.nbr_read = rd.p ? rd.as<int>() : P.nbr;
   };

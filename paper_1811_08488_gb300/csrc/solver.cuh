@@ -52,7 +52,7 @@ struct BlockPlan {
   int nrhs = 0;
   int Ls = 0;
   DevBuf nbr_oe, nbr_eo, gmap_b, gowner;
-  DevBuf nbr_read[2][4];  // BlockGeometry::nbr_read
+  DevBuf nbr_read[2][4];  // [snake][hop] present_neighbours, where a hop has needed them
   bool have_dense[2] = {false, false};
   DevBuf links;
   long long link_bstride = 0;
