@@ -408,12 +408,13 @@ __device__ __forceinline__ void ls_column_reg(R *T, const R *X, int Ls, bool dow
   for (int j = 0; j < LM; ++j)
     if (j == Ls - 1) last = v[j];
   R out_prev = v[0];
-  v[0] = p0 * v[0] - p1 * mf * last;
+  // (the larger term is the one that is not rounded before the sum)
+  v[0] = fma(p0, v[0], -p1 * mf * last);
 #pragma unroll
   for (int j = 1; j < LM; ++j)
     if (j < Ls) {
       const R t = v[j];
-      v[j] = p0 * t + p1 * out_prev;
+      v[j] = fma(p0, t, p1 * out_prev);
       out_prev = t;
     }
   if (X) {
@@ -455,8 +456,8 @@ __device__ __forceinline__ void ls_column_smem(R *T, const R *X, int Ls, bool do
   }
   const R p0 = c.p0q, p1 = c.p1q;
   const R last = T[ix(Ls - 1)];
-  for (int j = Ls - 1; j >= 1; --j) T[ix(j)] = p0 * T[ix(j)] + p1 * T[ix(j - 1)];
-  T[ix(0)] = p0 * T[ix(0)] - p1 * mf * last;
+  for (int j = Ls - 1; j >= 1; --j) T[ix(j)] = fma(p0, T[ix(j)], p1 * T[ix(j - 1)]);
+  T[ix(0)] = fma(p0, T[ix(0)], -p1 * mf * last);
   if (X) {
     const R a0 = c.a0, a1 = c.a1;
     for (int j = 1; j < Ls; ++j) T[ix(j)] += a0 * X[ix(j)] + a1 * X[ix(j - 1)];

@@ -79,7 +79,8 @@ __global__ void __launch_bounds__(128) ls2_kernel(char *out, const char *in, lon
 #pragma unroll
     for (int k = 0; k < 24; ++k) a0[k] = a1[k] = 0.f;
   }
-  ls_lanes<DAG>(a0, a1, inv != 0, Ls, np, jp, lane, cf.f, pair_lanes(lane, jp, np, cf.f.mf));
+  ls_lanes<DAG, true>(a0, a1, inv != 0, Ls, np, jp, lane, cf.f,
+                      pair_lanes(lane, jp, np, cf.f.mf));
   if (active) store24x2<F32>(out + rhs * rstride, 0, nsite * Ls, e, a0, a1);
 }
 
