@@ -95,7 +95,7 @@ __device__ __forceinline__ void adag_times(const Cx<R> w0, const Cx<R> w1, Cx<R>
   }
 }
 
-template <class R, int MU, bool FWD, bool DAG>
+template <class R, int MU, bool FWD, bool DAG, bool PRE>
 __device__ __forceinline__ void proj_mul_acc(R *acc, const R *v, const R *u);
 
 // One direction of the hop: project, multiply by U or U^+, reconstruct, add.
@@ -115,28 +115,32 @@ __device__ __forceinline__ void hop_dir(typename S::R *acc, const char *in, long
     const R fm = s == 0 ? -mf : (R)1;
     load12<S, true>(in, soff, cs, j * Ls + sm, w);
 #pragma unroll
-    for (int k = 0; k < 12; ++k) v[k] = b * v[k] + c * fm * w[k];
+    for (int k = 0; k < 12; ++k) v[k] = fma(b, v[k], c * fm * w[k]);
     const int sp = s == Ls - 1 ? 0 : s + 1;
     const R fp = s == Ls - 1 ? -mf : (R)1;
     load12<S, false>(in, soff, cs, j * Ls + sp, w);
 #pragma unroll
-    for (int k = 0; k < 12; ++k) v[12 + k] = b * v[12 + k] + c * fp * w[k];
+    for (int k = 0; k < 12; ++k) v[12 + k] = fma(b, v[12 + k], c * fp * w[k]);
   }
   R u[18];
   load_link<S>(lk, ls, u, RC ? 1 : 0);
-  proj_mul_acc<R, MU, FWD, DAG>(acc, v, u);
+  proj_mul_acc<R, MU, FWD, DAG, PRE>(acc, v, u);
 }
 
 // Project v with (1 - sg g_mu), multiply the two-spinor by U (forward) or U^+
 // (backward), reconstruct and add to acc. In FP64 the FP64 pipe is the bound
 // (a DFMA takes 65 cycles per warp and scheduler), so U h is a chain of 72
 // multiply-adds: `re += ur * hr - ui * hi` compiles to a product, a
-// multiply-add and a sum, 108 operations. Measured with M_phi taken out of the
-// hops (mphi_input) and whole warps (hop_sites_per_cta): A in FP64 on
-// 16^3 x 32 x 12 8.57 -> 5.58 ms, 0.69 of the FP64 pipe's rate; D_PC^+ in FP32
-// with Ls = 9 and three right-hand sides on 12 x 10 x 14 x 18 148 -> 119 us.
-template <class R, int MU, bool FWD, bool DAG>
+// multiply-add and a sum, 108 operations. Measured with M_phi taken out of D_PC's hops
+// (mphi_input) and whole warps (hop_sites_per_cta): A in FP64 on
+// 16^3 x 32 x 12 8.57 -> 5.58 ms, 0.69 of the FP64 pipe's rate. Its error, against 80-bit
+// arithmetic, is 0.94 to 0.98 of what it was for D_PC and A, 1.00 to 1.02 for one hop.
+// FP32 and FP16 (odd Ls) wait for their gather and take what has no larger error than
+// before: products summed in pairs with M_phi on load, the sums of Re U h and Im U h
+// apart otherwise. As one chain the error of one hop is 4 to 6 % larger.
+template <class R, int MU, bool FWD, bool DAG, bool PRE>
 __device__ __forceinline__ void proj_mul_acc(R *acc, const R *v, const R *u) {
+  constexpr bool kChain = std::is_same<R, double>::value, kPairs = !kChain && PRE;
   constexpr R sg = (FWD != DAG) ? (R)1 : (R)-1;  // projector (1 - sg g_mu)
   Cx<R> h[2][3];
 #pragma unroll
@@ -155,16 +159,32 @@ __device__ __forceinline__ void proj_mul_acc(R *acc, const R *v, const R *u) {
   for (int sp = 0; sp < 2; ++sp) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      R re, im;
+      R re, im, re2, im2;  // (the products with Re U and with Im U)
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
         // forward: U[a][b]; backward: conj(U[b][a])
         const R ur = FWD ? u[2 * (3 * a + b)] : u[2 * (3 * b + a)];
         const R ui = FWD ? u[2 * (3 * a + b) + 1] : -u[2 * (3 * b + a) + 1];
-        re = b == 0 ? ur * h[sp][b].re : fma(ur, h[sp][b].re, re);
-        re = fma(-ui, h[sp][b].im, re);
-        im = b == 0 ? ur * h[sp][b].im : fma(ur, h[sp][b].im, im);
-        im = fma(ui, h[sp][b].re, im);
+        const R hr = h[sp][b].re, hi = h[sp][b].im;
+        if constexpr (kChain) {
+          re = b == 0 ? ur * hr : fma(ur, hr, re);
+          re = fma(-ui, hi, re);
+          im = b == 0 ? ur * hi : fma(ur, hi, im);
+          im = fma(ui, hr, im);
+        } else if constexpr (kPairs) {
+          const R pr = fma(ur, hr, -ui * hi), pi = fma(ur, hi, ui * hr);
+          re = b == 0 ? pr : re + pr;
+          im = b == 0 ? pi : im + pi;
+        } else {
+          re = b == 0 ? ur * hr : fma(ur, hr, re);
+          re2 = b == 0 ? ui * hi : fma(ui, hi, re2);
+          im = b == 0 ? ur * hi : fma(ur, hi, im);
+          im2 = b == 0 ? ui * hr : fma(ui, hr, im2);
+        }
+      }
+      if constexpr (!kChain && !kPairs) {
+        re -= re2;
+        im += im2;
       }
       w[sp][a] = {re, im};
     }
@@ -370,11 +390,29 @@ __device__ __forceinline__ void hop_body(const HopParams &P) {
   }
 }
 
+// CTAs per SM: FP32 with M_phi on load has too many values for three (80 registers: it
+// spilled, and took 84.9 us instead of 70.9 on 16^3 x 32, Ls = 7; with 128 registers 65.8),
+// the others gain from the third (adjoint 96.8 -> 77.7 us). FP64 CTAs have at most 128
+// threads and their registers are left to the compiler.
 template <class S, bool DAG, bool PRE, bool RC>
-__global__ void __launch_bounds__(256) hop_kernel(const __grid_constant__ HopParams P) {
+__global__ void __launch_bounds__(256, std::is_same<S, F32>::value &&PRE ? 2 : 3)
+    hop_kernel(const __grid_constant__ HopParams P) {
   prof_enter(P);
   hop_body<S, DAG, PRE, RC>(P);
   prof_exit(P);
+}
+template <bool DAG, bool PRE>
+__global__ void __launch_bounds__(256) hop64_kernel(const __grid_constant__ HopParams P) {
+  prof_enter(P);
+  hop_body<F64, DAG, PRE, false>(P);
+  prof_exit(P);
+}
+template <class S, bool DAG, bool PRE, bool RC>
+static constexpr auto hop_entry() {
+  if constexpr (std::is_same<S, F64>::value)
+    return hop64_kernel<DAG, PRE>;
+  else
+    return hop_kernel<S, DAG, PRE, RC>;
 }
 
 constexpr int kHopCtas = 4;  // CTAs of hop2_kernel per SM (128 registers a thread)
@@ -878,13 +916,16 @@ int sm_count() {
 // Two slices per thread for FP32/FP16/BF16 with even Ls; one otherwise.
 static bool hop_pairs(int Ls, dwf_prec p) { return p != DWF_FP64 && Ls % 2 == 0; }
 
-// Sites per CTA. The one-slice kernel takes, between a half and a whole of its
-// largest CTA, the number of sites that leaves the fewest idle lanes in the last
-// warp: a warp instruction of the FP64 pipe takes as long with idle lanes (Ls =
-// 12: 8 sites fill three warps, 10 sites leave 8 of 128 lanes idle).
+// Sites per CTA. The one-slice kernel takes as many as its largest CTA holds; in FP64,
+// between a half and a whole of that, the number that leaves the fewest idle lanes in the
+// last warp: a warp instruction of the FP64 pipe takes as long with idle lanes (Ls =
+// 12: 8 sites fill three warps, 10 sites leave 8 of 128 lanes idle). For the other types,
+// which wait for the gather, that made more CTAs for nothing (12 x 10 x 14 x 18, Ls = 7,
+// FP16 adjoint: 22.7 against 18.7 us).
 int hop_sites_per_cta(int Ls, dwf_prec p) {
   if (hop_pairs(Ls, p)) return 4 * (32 / (Ls / 2));  // four warps of whole sites
   const int most = (p == DWF_FP64 ? 128 : 256) / Ls;
+  if (p != DWF_FP64) return most;
   int best = most;
   auto lanes = [&](int n) { return (n * Ls + 31) / 32 * 32; };
   for (int n = most; n >= 1 && 2 * n >= most; --n)
@@ -990,7 +1031,7 @@ static void launch_t(const HopParams &P0, int nrhs, cudaStream_t st, dwf_prec pr
     }
   }
   dim3 block((nsites * P.Ls + 31) / 32 * 32);
-  hop_kernel<S, DAG, PRE, RC><<<grid, block, smem, st>>>(P);
+  hop_entry<S, DAG, PRE, RC>()<<<grid, block, smem, st>>>(P);
   DWF_CUDA_TRY(cudaGetLastError());
 }
 
@@ -1034,13 +1075,13 @@ static void allow_big_smem(K *kernel) {
 }
 template <class S>
 static void prepare_one() {
-  allow_big_smem(hop_kernel<S, false, false, false>);
-  allow_big_smem(hop_kernel<S, false, true, false>);
-  allow_big_smem(hop_kernel<S, true, false, false>);
+  allow_big_smem(hop_entry<S, false, false, false>());
+  allow_big_smem(hop_entry<S, false, true, false>());
+  allow_big_smem(hop_entry<S, true, false, false>());
   if constexpr (!std::is_same<S, F64>::value) {
-    allow_big_smem(hop_kernel<S, false, false, true>);
-    allow_big_smem(hop_kernel<S, false, true, true>);
-    allow_big_smem(hop_kernel<S, true, false, true>);
+    allow_big_smem(hop_entry<S, false, false, true>());
+    allow_big_smem(hop_entry<S, false, true, true>());
+    allow_big_smem(hop_entry<S, true, false, true>());
   }
 }
 void prepare_kernels() {
