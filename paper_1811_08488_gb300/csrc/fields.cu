@@ -179,6 +179,12 @@ constexpr int kIoElems = 128;
 template <class C> __host__ __device__ inline int io_row(int sites) {  // bytes of one s
   return sites * 24 * (int)sizeof(C) + 16;
 }
+// The thread's next word of the tile's canonical side, kIoElems further on: words of
+// slice s, then of the next one. (A loop over the slices, each with a part of the
+// CTA, took a CTA of few sites longer: 4^4, Ls = 32, 8.4 us instead of 6.4 the direct way.)
+__device__ __forceinline__ void io_next(int &s, int &w, int words) {
+  for (w += kIoElems; w >= words; w -= words) ++s;
+}
 template <class S, class C>
 __global__ void __launch_bounds__(kIoElems) import_tile_kernel(char *native, long long nstride,
                                                                long long soff, const C *canon,
@@ -186,14 +192,13 @@ __global__ void __launch_bounds__(kIoElems) import_tile_kernel(char *native, lon
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int rhs = blockIdx.y, h0 = blockIdx.x * sites, nh = min(sites, nsite - h0);
   const int row = io_row<C>(sites), words = nh * 24 * (int)sizeof(C) / 16;
-  for (int s = 0; s < Ls; ++s) {
+  for (int s = threadIdx.x / words, w = threadIdx.x % words; s < Ls; io_next(s, w, words)) {
     const uint4 *src = reinterpret_cast<const uint4 *>(
         canon + (((size_t)rhs * Ls + s) * nsite + h0) * 24);
-    for (int w = threadIdx.x; w < words; w += kIoElems)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                       static_cast<uint32_t>(__cvta_generic_to_shared(smem_raw + s * row + w * 16))),
-                   "l"(src + w)
-                   : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(smem_raw + s * row + w * 16))),
+                 "l"(src + w)
+                 : "memory");
   }
   asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
   __syncthreads();
@@ -238,10 +243,9 @@ __global__ void __launch_bounds__(kIoElems) export_tile_kernel(C *canon, const c
     }
   }
   __syncthreads();
-  for (int s = 0; s < Ls; ++s) {
+  for (int s = threadIdx.x / words, w = threadIdx.x % words; s < Ls; io_next(s, w, words)) {
     uint4 *dst = reinterpret_cast<uint4 *>(canon + (((size_t)rhs * Ls + s) * nsite + h0) * 24);
-    for (int w = threadIdx.x; w < words; w += kIoElems)
-      dst[w] = *reinterpret_cast<const uint4 *>(smem_raw + s * row + w * 16);
+    dst[w] = *reinterpret_cast<const uint4 *>(smem_raw + s * row + w * 16);
   }
 }
 
