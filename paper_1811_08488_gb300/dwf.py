@@ -179,7 +179,9 @@ _current_stream = None  # torch.cuda.current_stream, once torch is needed
 def _stream(stream):
     global _current_stream
     if stream is not None:
-        return stream
+        # (c_void_p refuses what is no integer; as an argument type it would take
+        # bytes, text and objects with _as_parameter_ for the pointer)
+        return stream if type(stream) is int else C.c_void_p(stream)
     if _current_stream is None:
         import torch
         _current_stream = torch.cuda.current_stream
