@@ -378,6 +378,17 @@ __device__ __forceinline__ const LsK<R> &kc(const LsCoef &c) {
     return c.d;
 }
 
+// p0 y + q z. FP32: the larger term is the one that is not rounded before the sum. FP64:
+// as the compiler contracts it (M_5 of small fields 14.7 us, the other way 16.5).
+template <class R>
+struct MixSlices {
+  R p0;
+  __device__ __forceinline__ R operator()(R y, R q, R z) const {
+    if constexpr (std::is_same<R, float>::value) return fma(p0, y, q * z);
+    else return p0 * y + q * z;
+  }
+};
+
 // The column is first read into registers (LM >= Ls, loops unrolled over LM
 // with j < Ls guards, so no register array is indexed at run time) and the
 // recursions run there; shared memory is read once and written once.
@@ -408,13 +419,13 @@ __device__ __forceinline__ void ls_column_reg(R *T, const R *X, int Ls, bool dow
   for (int j = 0; j < LM; ++j)
     if (j == Ls - 1) last = v[j];
   R out_prev = v[0];
-  // (the larger term is the one that is not rounded before the sum)
-  v[0] = fma(p0, v[0], -p1 * mf * last);
+  const MixSlices<R> mix{p0};
+  v[0] = mix(v[0], -p1 * mf, last);
 #pragma unroll
   for (int j = 1; j < LM; ++j)
     if (j < Ls) {
       const R t = v[j];
-      v[j] = fma(p0, t, p1 * out_prev);
+      v[j] = mix(t, p1, out_prev);
       out_prev = t;
     }
   if (X) {
@@ -456,8 +467,9 @@ __device__ __forceinline__ void ls_column_smem(R *T, const R *X, int Ls, bool do
   }
   const R p0 = c.p0q, p1 = c.p1q;
   const R last = T[ix(Ls - 1)];
-  for (int j = Ls - 1; j >= 1; --j) T[ix(j)] = fma(p0, T[ix(j)], p1 * T[ix(j - 1)]);
-  T[ix(0)] = fma(p0, T[ix(0)], -p1 * mf * last);
+  const MixSlices<R> mix{p0};
+  for (int j = Ls - 1; j >= 1; --j) T[ix(j)] = mix(T[ix(j)], p1, T[ix(j - 1)]);
+  T[ix(0)] = mix(T[ix(0)], -p1 * mf, last);
   if (X) {
     const R a0 = c.a0, a1 = c.a1;
     for (int j = 1; j < Ls; ++j) T[ix(j)] += a0 * X[ix(j)] + a1 * X[ix(j - 1)];
