@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kEigThreads) gram_kernel(const GramArgs a) {
   if (threadIdx.x == 0) a.counters[tile] = 0u;
 }
 
-// Few Y vectors (ny <= NJ <= 4) against many X, one of them not FP32:
+// Few Y vectors (ny <= NJ <= 4) against many X (what gram_stream does not take):
 // the 8 warps of a CTA walk the same stretch of 32 elements (groups of 4 reals
 // or 16-byte chunks of 8 reals), warp w taking X vectors
 // ibase + w + 8 t (t < NI) and every Y vector, so each X vector is read once
@@ -313,6 +313,26 @@ __global__ void __launch_bounds__(kEigThreads) gram_skinny_kernel(const GramArgs
   if (threadIdx.x == 0) a.counters[tile] = 0u;
 }
 
+// The sums over the warp of N values per lane (N a power of two up to 32): lane l ends
+// with value l / (32 / N). Each step exchanges half of the values that are left, so it
+// takes N - 1 additions and a few more instead of 5 N: FP64 additions are what the ends
+// of the multi-dots wait for (65 cycles per warp and scheduler).
+template <int N>
+__device__ __forceinline__ double warp_sums(double (&d)[N], int lane) {
+  int o = 16;
+#pragma unroll
+  for (int half = N / 2; half > 0; half /= 2, o /= 2) {
+    const bool upper = lane & o;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const double send = upper ? d[i] : d[i + half], keep = upper ? d[i + half] : d[i];
+      d[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  for (; o > 0; o /= 2) d[0] += __shfl_xor_sync(0xffffffffu, d[0], o);
+  return d[0];
+}
+
 // FP32 X against few FP32 Y (ny <= NJ): the fields are flat arrays, so the CTA streams
 // segments of 64 float4 of 8 NI vectors X and of every Y through a ring of stages in
 // shared memory (cp.async, kStreamBytes of them in flight per CTA), and warp w
@@ -330,7 +350,8 @@ template <int NI, int NJ> constexpr int stream_stages() {
 
 template <int NI, int NJ>
 __global__ void __launch_bounds__(kEigThreads, 2) gram_stream_kernel(const GramArgs a) {
-  constexpr int NV = 8 * NI * NJ * 2, NVEC = 8 * NI + NJ, kStages = stream_stages<NI, NJ>();
+  constexpr int NW = NI * NJ * 2, NV = 8 * NW, NVEC = 8 * NI + NJ, kStages = stream_stages<NI, NJ>();
+  constexpr int NB = NW <= 2 ? 2 : NW <= 4 ? 4 : 8;  // values summed at a time
   static_assert(NV <= kMaxValues, "too many partial sums per CTA");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_last;
@@ -401,20 +422,19 @@ __global__ void __launch_bounds__(kEigThreads, 2) gram_stream_kernel(const GramA
     stage = stage + 1 == kStages ? 0 : stage + 1;
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
-  // value v = ((w NI + t) NJ + j) 2 + c: warp sums, written by lane 0 of warp w
+  // value v = ((w NI + t) NJ + j) 2 + c = w NW + i: warp sums
   double *part = a.partials + (size_t)tile * gridDim.x * NV;
+  const int vi = lane / (32 / NB);  // of every NB values, the one that this lane ends with
+  const bool mine = lane % (32 / NB) == 0;
 #pragma unroll
-  for (int t = 0; t < NI; ++t)
+  for (int b = 0; b < NW; b += NB) {
+    double d[NB];
 #pragma unroll
-    for (int j = 0; j < NJ; ++j)
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        double d = acc[t][j][c].value();
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
-        if (lane == 0)
-          part[(size_t)(((w * NI + t) * NJ + j) * 2 + c) * gridDim.x + blockIdx.x] = d;
-      }
+    for (int i = 0; i < NB; ++i)
+      d[i] = b + i < NW ? acc[(b + i) / (2 * NJ)][(b + i) / 2 % NJ][i % 2].value() : 0.0;
+    const double sum = warp_sums(d, lane);
+    if (mine && b + vi < NW) part[(size_t)(w * NW + b + vi) * gridDim.x + blockIdx.x] = sum;
+  }
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -424,17 +444,22 @@ __global__ void __launch_bounds__(kEigThreads, 2) gram_stream_kernel(const GramA
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  // the last CTA: a warp per value, in a fixed order
-  for (int v = w; v < NV; v += kEigThreads / 32) {
-    const volatile double *vp = part + (size_t)v * gridDim.x;
-    double sum = 0.0;
-    for (unsigned int k = lane; k < gridDim.x; k += 32) sum += vp[k];
+  // the last CTA: each warp its own values, in a fixed order
+#pragma unroll 1
+  for (int b = 0; b < NW; b += NB) {
+    double d[NB];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
-    const int c = v & 1, j = (v >> 1) % NJ, wt = (v >> 1) / NJ;
-    const int gi = ibase + wt / NI + 8 * (wt % NI);
-    if (lane == 0 && gi < a.nx && j < a.ny)
-      reinterpret_cast<double *>(a.G + (size_t)gi * a.ldg + j)[c] = sum;
+    for (int i = 0; i < NB; ++i) d[i] = 0.0;
+    for (unsigned int k = lane; k < gridDim.x; k += 32) {
+      const double *p = part + (size_t)(w * NW + b) * gridDim.x + k;
+#pragma unroll
+      for (int i = 0; i < NB; ++i)
+        if (b + i < NW) d[i] += __ldcg(p + (size_t)i * gridDim.x);
+    }
+    const double sum = warp_sums(d, lane);
+    const int v = b + vi, gi = ibase + w + 8 * (v / (2 * NJ)), gj = v / 2 % NJ;
+    if (mine && v < NW && gi < a.nx && gj < a.ny)
+      reinterpret_cast<double *>(a.G + (size_t)gi * a.ldg + gj)[v % 2] = sum;
   }
   if (threadIdx.x == 0) a.counters[tile] = 0u;
 }
@@ -449,14 +474,16 @@ static void gram_stream_go(const GramArgs &a, cudaStream_t st) {
   gram_stream_kernel<NI, NJ><<<grid, kEigThreads, bytes, st>>>(a);
   DWF_CUDA_TRY(cudaGetLastError());
 }
-// All X in one tile of up to 32 vectors, so that the Y are read once.
+// All X in one tile of up to 32 vectors, so that the Y are read once; more of them in
+// tiles of about the same number.
 template <int NJ>
 static void gram_stream(const GramArgs &a, cudaStream_t st) {
-  if (a.nx <= 8)
+  const int tiles = (a.nx + 31) / 32, ni = (a.nx + 8 * tiles - 1) / (8 * tiles);
+  if (ni == 1)
     gram_stream_go<1, NJ>(a, st);
-  else if (a.nx <= 16)
+  else if (ni == 2)
     gram_stream_go<2, NJ>(a, st);
-  else if (a.nx <= 24)
+  else if (ni == 3)
     gram_stream_go<3, NJ>(a, st);
   else
     gram_stream_go<4, NJ>(a, st);
@@ -477,7 +504,8 @@ static void gram_skinny_launch(const GramArgs &a, dwf_prec xprec, dwf_prec yprec
     yprec == DWF_FP64 ? gram_skinny_go<NI, NJ, F16, F64>(a, st)
                       : gram_skinny_go<NI, NJ, F16, F32>(a, st);
   else
-    gram_skinny_go<NI, NJ, F32, F64>(a, st);  // (FP32 Y: gram_stream)
+    yprec == DWF_FP64 ? gram_skinny_go<NI, NJ, F32, F64>(a, st)
+                      : gram_skinny_go<NI, NJ, F32, F32>(a, st);
 }
 
 template <int TI, int TJ>
@@ -517,7 +545,12 @@ void gram(const VecSet &X, const VecSet &Y, long long cs, double2 *G, int ldg,
   a.ldg = ldg;
   a.partials = w.partials;
   a.counters = w.counters;
-  if (Y.n <= 4 && X.prec == DWF_FP32 && Y.prec == DWF_FP32) {
+  // Streaming takes longer for one long Y against more than 24 X (the ring's barriers for
+  // few products; 32 and 64 X on 16^3 x 32 x 12: 816 and 1528 us against 838 and 1587), and
+  // for vectors of a few dozen segments against many X (the ends of the CTAs, which
+  // gram_skinny spreads over tiles; 32 X, 3 Y on 4^4 x 4: deflation 57 against 65 us).
+  const bool few = (Y.n == 1 && X.n > 24 && a.n4 >= 1 << 20) || (X.n > 16 && a.n4 < 64 * kSeg);
+  if (Y.n <= 4 && X.prec == DWF_FP32 && Y.prec == DWF_FP32 && !few) {
     if (Y.n == 1)
       gram_stream<1>(a, st);
     else if (Y.n == 2)
