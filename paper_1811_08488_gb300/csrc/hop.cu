@@ -20,14 +20,14 @@
 //   has just freed, while the projected spins are multiplied by the link.
 // And the Ls epilogue's scan runs one step over all 24 components at a time, with
 // shared factors, 480 instead of about 1100 instructions per thread.
-// Measured on 24^3 x 64 x 16, before -> after: FP32 M^4 613 -> 533 us, adjoint
-// 513 -> 410, FP16 642 -> 486 and 433 -> 384, A in FP32 2547 -> 2072. Not kept:
+// Measured on 24^3 x 64 x 16, before -> now: FP32 M^4 613 -> 504 us, adjoint
+// 513 -> 397, FP16 642 -> 483 and 433 -> 373. Not kept:
 // rings of stages in shared memory filled by cp.async or by TMA boxes, all
 // bit-identical: the work to issue them (150 instructions a direction beside 230 of
 // arithmetic) and the larger code cost more than the waiting they save (853 and
 // 883 us for FP32 M^4); mma.m16n8k16 for FP16 fields (one site per warp: 968
 // instructions per site instead of 553, 660 us for the adjoint); an L2 prefetch
-// of the rows that come next (535 us).
+// of the rows that come next (FP32 M^4 631 us, adjoint 535).
 //
 // The other form of the kernel (DENSE = false) runs direction by direction, leaves out
 // those that no lane has, and reads the links where they are: for the outer ring of a
@@ -95,12 +95,12 @@ __device__ __forceinline__ void adag_times(const Cx<R> w0, const Cx<R> w1, Cx<R>
   }
 }
 
-template <class R, int MU, bool FWD, bool DAG, bool PRE>
+template <class R, int MU, bool FWD, bool DAG, bool PAIRS>
 __device__ __forceinline__ void proj_mul_acc(R *acc, const R *v, const R *u);
 
 // One direction of the hop: project, multiply by U or U^+, reconstruct, add.
 // `lk` is the link record.
-template <class S, int MU, bool FWD, bool DAG, bool PRE, bool RC>
+template <class S, int MU, bool FWD, bool DAG, bool PRE, bool RC, bool PAIRS>
 __device__ __forceinline__ void hop_dir(typename S::R *acc, const char *in, long long soff,
                                         int cs, int j, int s, int Ls, const uint4 *lk,
                                         size_t ls, const LsCoef &cf) {
@@ -124,7 +124,7 @@ __device__ __forceinline__ void hop_dir(typename S::R *acc, const char *in, long
   }
   R u[18];
   load_link<S>(lk, ls, u, RC ? 1 : 0);
-  proj_mul_acc<R, MU, FWD, DAG, PRE>(acc, v, u);
+  proj_mul_acc<R, MU, FWD, DAG, PAIRS>(acc, v, u);
 }
 
 // Project v with (1 - sg g_mu), multiply the two-spinor by U (forward) or U^+
@@ -133,14 +133,15 @@ __device__ __forceinline__ void hop_dir(typename S::R *acc, const char *in, long
 // multiply-adds: `re += ur * hr - ui * hi` compiles to a product, a
 // multiply-add and a sum, 108 operations. Measured with M_phi taken out of D_PC's hops
 // (mphi_input) and whole warps (hop_sites_per_cta): A in FP64 on
-// 16^3 x 32 x 12 8.57 -> 5.58 ms, 0.69 of the FP64 pipe's rate. Its error, against 80-bit
-// arithmetic, is 0.94 to 0.98 of what it was for D_PC and A, 1.00 to 1.02 for one hop.
+// 16^3 x 32 x 12 8.57 -> 5.59 ms, 0.69 of the FP64 pipe's rate. Its error, against 80-bit
+// arithmetic, is 0.94 to 0.98 of what it was for D_PC and A. A single hop has nothing to
+// make up for the chain's 1 to 2 %: its products are summed in pairs (PAIRS).
 // FP32 and FP16 (odd Ls) wait for their gather and take what has no larger error than
-// before: products summed in pairs with M_phi on load, the sums of Re U h and Im U h
-// apart otherwise. As one chain the error of one hop is 4 to 6 % larger.
-template <class R, int MU, bool FWD, bool DAG, bool PRE>
+// before: pairs with M_phi on load, the sums of Re U h and Im U h apart otherwise. As
+// one chain the error of one hop is 4 to 6 % larger.
+template <class R, int MU, bool FWD, bool DAG, bool PAIRS>
 __device__ __forceinline__ void proj_mul_acc(R *acc, const R *v, const R *u) {
-  constexpr bool kChain = std::is_same<R, double>::value, kPairs = !kChain && PRE;
+  constexpr bool kChain = std::is_same<R, double>::value && !PAIRS;
   constexpr R sg = (FWD != DAG) ? (R)1 : (R)-1;  // projector (1 - sg g_mu)
   Cx<R> h[2][3];
 #pragma unroll
@@ -171,7 +172,7 @@ __device__ __forceinline__ void proj_mul_acc(R *acc, const R *v, const R *u) {
           re = fma(-ui, hi, re);
           im = b == 0 ? ur * hi : fma(ur, hi, im);
           im = fma(ui, hr, im);
-        } else if constexpr (kPairs) {
+        } else if constexpr (PAIRS) {
           const R pr = fma(ur, hr, -ui * hi), pi = fma(ur, hi, ui * hr);
           re = b == 0 ? pr : re + pr;
           im = b == 0 ? pi : im + pi;
@@ -182,7 +183,7 @@ __device__ __forceinline__ void proj_mul_acc(R *acc, const R *v, const R *u) {
           im2 = b == 0 ? ui * hr : fma(ui, hr, im2);
         }
       }
-      if constexpr (!kChain && !kPairs) {
+      if constexpr (!kChain && !PAIRS) {
         re -= re2;
         im += im2;
       }
@@ -204,7 +205,7 @@ __device__ __forceinline__ void proj_mul_acc(R *acc, const R *v, const R *u) {
   }
 }
 
-template <class S, int MU, bool DAG, bool PRE, bool RC>
+template <class S, int MU, bool DAG, bool PRE, bool RC, bool PAIRS>
 __device__ __forceinline__ void hop_mu(typename S::R *acc, const HopParams &P, const char *in,
                                        const uint4 *links, const int *nb, int site, int s,
                                        const LsCoef &cf) {
@@ -213,10 +214,10 @@ __device__ __forceinline__ void hop_mu(typename S::R *acc, const HopParams &P, c
   const size_t ls = (size_t)P.link_cs;
   const uint4 *lmu = links + (size_t)MU * LC * ls;
   if (jf >= 0 && jf < P.in_limit)
-    hop_dir<S, MU, true, DAG, PRE, RC>(acc, in, P.in.scale_off, P.in.cs, jf, s, P.Ls,
+    hop_dir<S, MU, true, DAG, PRE, RC, PAIRS>(acc, in, P.in.scale_off, P.in.cs, jf, s, P.Ls,
                                    lmu + P.out_link_off + site, ls, cf);
   if (jb >= 0 && jb < P.in_limit)
-    hop_dir<S, MU, false, DAG, PRE, RC>(acc, in, P.in.scale_off, P.in.cs, jb, s, P.Ls,
+    hop_dir<S, MU, false, DAG, PRE, RC, PAIRS>(acc, in, P.in.scale_off, P.in.cs, jb, s, P.Ls,
                                     lmu + P.in_link_off + jb, ls, cf);
 }
 
@@ -310,8 +311,9 @@ __device__ __noinline__ void prof_exit(const HopParams &P) {
   __threadfence();
 }
 
-// One thread per output (site, s): used for FP64 fields and odd Ls.
-template <class S, bool DAG, bool PRE, bool RC>
+// One thread per output (site, s): used for FP64 fields and odd Ls. PAIRS: how U h is summed
+// (proj_mul_acc).
+template <class S, bool DAG, bool PRE, bool RC, bool PAIRS>
 __device__ __forceinline__ void hop_body(const HopParams &P) {
   using R = typename S::R;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -337,10 +339,10 @@ __device__ __forceinline__ void hop_body(const HopParams &P) {
   for (int k = 0; k < 24; ++k) acc[k] = 0;
   if (active) {
     const int *nb = P.nbr + (size_t)site * 8;
-    hop_mu<S, 0, DAG, PRE, RC>(acc, P, in, links, nb, site, s, cf);
-    hop_mu<S, 1, DAG, PRE, RC>(acc, P, in, links, nb, site, s, cf);
-    hop_mu<S, 2, DAG, PRE, RC>(acc, P, in, links, nb, site, s, cf);
-    hop_mu<S, 3, DAG, PRE, RC>(acc, P, in, links, nb, site, s, cf);
+    hop_mu<S, 0, DAG, PRE, RC, PAIRS>(acc, P, in, links, nb, site, s, cf);
+    hop_mu<S, 1, DAG, PRE, RC, PAIRS>(acc, P, in, links, nb, site, s, cf);
+    hop_mu<S, 2, DAG, PRE, RC, PAIRS>(acc, P, in, links, nb, site, s, cf);
+    hop_mu<S, 3, DAG, PRE, RC, PAIRS>(acc, P, in, links, nb, site, s, cf);
   }
   const int e = site * Ls + s;
 
@@ -398,19 +400,20 @@ template <class S, bool DAG, bool PRE, bool RC>
 __global__ void __launch_bounds__(256, std::is_same<S, F32>::value &&PRE ? 2 : 3)
     hop_kernel(const __grid_constant__ HopParams P) {
   prof_enter(P);
-  hop_body<S, DAG, PRE, RC>(P);
+  hop_body<S, DAG, PRE, RC, PRE>(P);
   prof_exit(P);
 }
-template <bool DAG, bool PRE>
+template <bool DAG, bool PRE, bool PAIRS>
 __global__ void __launch_bounds__(256) hop64_kernel(const __grid_constant__ HopParams P) {
   prof_enter(P);
-  hop_body<F64, DAG, PRE, false>(P);
+  hop_body<F64, DAG, PRE, false, PAIRS>(P);
   prof_exit(P);
 }
+// single: the hop is the whole operator (FP64: summed in pairs, see proj_mul_acc)
 template <class S, bool DAG, bool PRE, bool RC>
-static constexpr auto hop_entry() {
+static auto hop_entry(bool single) {
   if constexpr (std::is_same<S, F64>::value)
-    return hop64_kernel<DAG, PRE>;
+    return PRE || single ? hop64_kernel<DAG, PRE, true> : hop64_kernel<DAG, PRE, PRE>;
   else
     return hop_kernel<S, DAG, PRE, RC>;
 }
@@ -1031,7 +1034,7 @@ static void launch_t(const HopParams &P0, int nrhs, cudaStream_t st, dwf_prec pr
     }
   }
   dim3 block((nsites * P.Ls + 31) / 32 * 32);
-  hop_entry<S, DAG, PRE, RC>()<<<grid, block, smem, st>>>(P);
+  hop_entry<S, DAG, PRE, RC>(!P.inv && !P.has_x)<<<grid, block, smem, st>>>(P);
   DWF_CUDA_TRY(cudaGetLastError());
 }
 
@@ -1075,13 +1078,15 @@ static void allow_big_smem(K *kernel) {
 }
 template <class S>
 static void prepare_one() {
-  allow_big_smem(hop_entry<S, false, false, false>());
-  allow_big_smem(hop_entry<S, false, true, false>());
-  allow_big_smem(hop_entry<S, true, false, false>());
-  if constexpr (!std::is_same<S, F64>::value) {
-    allow_big_smem(hop_entry<S, false, false, true>());
-    allow_big_smem(hop_entry<S, false, true, true>());
-    allow_big_smem(hop_entry<S, true, false, true>());
+  for (bool single : {false, true}) {
+    allow_big_smem(hop_entry<S, false, false, false>(single));
+    allow_big_smem(hop_entry<S, false, true, false>(single));
+    allow_big_smem(hop_entry<S, true, false, false>(single));
+    if constexpr (!std::is_same<S, F64>::value) {
+      allow_big_smem(hop_entry<S, false, false, true>(single));
+      allow_big_smem(hop_entry<S, false, true, true>(single));
+      allow_big_smem(hop_entry<S, true, false, true>(single));
+    }
   }
 }
 void prepare_kernels() {
