@@ -186,7 +186,8 @@ typedef struct {
 /* Device time of one hop-kernel family, from dwf_profile_read. */
 typedef struct {
   char name[48];       /* kernel and template arguments, e.g.
-                        * "hop2_kernel<F16,1,0,0,1>" (S, DAG, PRE, RECON, EPI) */
+                        * "hop2_kernel<F16,1,0,0,1>" (S, DAG, PRE, RECON, EPI;
+                        * with and without staged links together)              */
   long long launches;  /* launches since profiling was (re)enabled            */
   double seconds;      /* sum over launches of (exit of the last CTA to
                         * finish - entry of CTA 0), from the global timer     */

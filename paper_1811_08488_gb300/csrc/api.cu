@@ -354,8 +354,9 @@ dwf_status dwf_odd_reconstruct(dwf_ctx *ctx, void *psi_odd, const void *psi_even
 
 // Name of the kernel behind profiler slot `slot` (role * 32 + prec * 8 + DAG * 4
 // + PRE * 2 + EPI) in this context: hop2_kernel for FP32/FP16/BF16 with even
-// Ls, hop_kernel otherwise; the template arguments as the kernel declares
-// them, and " [block]" for launches of the block operator A_s.
+// Ls, hop_kernel (hop64_kernel in FP64) otherwise; its template arguments without
+// hop2_kernel's DENSE (both forms of a hop are one entry), and " [block]" for
+// launches of the block operator A_s.
 static std::string prof_slot_name(const dwf_ctx *ctx, int slot) {
   static const char *kS[4] = {"F64", "F32", "F16", "BF16"};
   const int role = slot / 32;

@@ -393,8 +393,8 @@ __device__ __forceinline__ void hop_body(const HopParams &P) {
 }
 
 // CTAs per SM: FP32 with M_phi on load has too many values for three (80 registers: it
-// spilled, and took 84.9 us instead of 70.9 on 16^3 x 32, Ls = 7; with 128 registers 65.8),
-// the others gain from the third (adjoint 96.8 -> 77.7 us). FP64 CTAs have at most 128
+// spilled, and took 84.9 us instead of 70.9 on 16^3 x 32, Ls = 7; with 128 registers 66.7),
+// the others gain from the third (adjoint 96.8 -> 78.0 us). FP64 CTAs have at most 128
 // threads and their registers are left to the compiler.
 template <class S, bool DAG, bool PRE, bool RC>
 __global__ void __launch_bounds__(256, std::is_same<S, F32>::value &&PRE ? 2 : 3)

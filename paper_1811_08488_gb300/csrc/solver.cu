@@ -110,12 +110,14 @@ void apply_dslash(dwf_ctx *ctx, void *out, const void *in, int out_parity, int d
   launch(ctx, p, P, dagger, dagger ? 0 : 1, nrhs, st);
 }
 
-// The input of a hop with M_phi: FP64 fields take M_phi in one Ls pass into
-// phi_tmp (returned; the hop then runs without it), others take it on load
-// (`in` is returned). On load every neighbour's M_phi costs 48 operations for
-// each of the 8 directions; in FP32 that is cheaper than a pass over the
-// field, on GB300's small FP64 pipe it is not (16^3 x 32 x 12, first hop of
-// D_PC: 384 of 1250 FP64 operations per element against 48 and 302 MB).
+// The input of a hop with M_phi inside an operator that has a temporary: FP64 fields
+// take M_phi in one Ls pass into phi_tmp (returned; the hop then runs without it),
+// others take it on load (`in` is returned). On load every neighbour's M_phi costs
+// 48 operations for each of the 8 directions; in FP32 that is cheaper than a pass over
+// the field, on GB300's small FP64 pipe it is not (16^3 x 32 x 12, first hop of
+// D_PC: 384 of 1250 FP64 operations per element against 48 and 302 MB). The single hop
+// (apply_dslash), which has no temporary, takes M_phi on load in FP64 too, and the
+// Shamir action (M_phi = 1) takes the pass as a copy.
 static const void *mphi_input(dwf_ctx *ctx, const void *in, char *phi_tmp, dwf_prec p, int nrhs,
                               const double *mf, const int *skip, cudaStream_t st) {
   if (p != DWF_FP64) return in;
